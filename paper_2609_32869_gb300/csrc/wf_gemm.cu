@@ -35,6 +35,7 @@
 #include <algorithm>
 
 #include "wf_device.cuh"
+#include "wf_gemm_epi.cuh"
 #include "wf_internal.h"
 
 namespace wf {
@@ -51,23 +52,12 @@ constexpr int kSmemBudgetLn = 110 * 1024;  // LN mode: resident token tiles + we
 constexpr int kMaxBT = 128;                // token rows per tile (MMA N)
 constexpr size_t kSmemPerSM = 228 * 1024;  // shared memory of one SM
 constexpr int kLnFuseMaxM = 256;              // token rows up to which LN is fused
+// Token rows above which pairs of SMs take a projection: at 288 rows (32
+// sequences) they halve most launches (fc2 33 -> 17 us, fc1 20 -> 13), while
+// up to 256 rows one token tile covers every row and only split-K over
+// clusters fills the GPU.
+constexpr int kWideMinM = 256;
 constexpr int kFoldMinTiles = 64;             // output tiles from which split-K folds into one CTA
-
-__device__ __forceinline__ void head_combine(float &m, float &s, int &arg, float &gm, int &garg,
-                                             float m2, float s2, int arg2, float gm2, int garg2) {
-  const float M = fmaxf(m, m2);
-  float ns = 0.f;
-  if (M != -INFINITY) {
-    ns = (m == -INFINITY ? 0.f : s * __expf(m - M)) + (m2 == -INFINITY ? 0.f : s2 * __expf(m2 - M));
-  }
-  if (m2 > m || (m2 == m && arg2 < arg)) arg = arg2;
-  m = M;
-  s = ns;
-  if (gm2 > gm || (gm2 == gm && garg2 < garg)) {
-    gm = gm2;
-    garg = garg2;
-  }
-}
 
 // Epilogue of 16 consecutive token columns t0..t0+15 for output feature n.
 // acc[] holds the 16 accumulated values; every global load of the chunk (the
@@ -128,90 +118,6 @@ __device__ __forceinline__ void epi_chunk(const GemmParams &p, int t0, int n, fl
       dst[((static_cast<size_t>(sp.x) * p.n_heads + h) * p.ctx + sp.y) * 64 + dd] =
           __float2bfloat16(acc[jj] + bn);
     }
-  }
-}
-
-// Four floats as four bf16 (round to nearest even) in one 8-byte word.
-__device__ __forceinline__ uint2 pack4_bf16(const float (&v)[4]) {
-  __nv_bfloat162 h[2] = {__floats2bfloat162_rn(v[0], v[1]), __floats2bfloat162_rn(v[2], v[3])};
-  return *reinterpret_cast<const uint2 *>(h);
-}
-// Non-residual epilogues of four features: GELU, then fp32, bf16 or the
-// query / key / value split with the cache scatter.
-template <int EPI>
-__device__ __forceinline__ void epi_quad_out(const GemmParams &p, int t, int n, float (&v)[4],
-                                             const int2 *tok_local, float (&fin)[4]) {
-  if constexpr (EPI == EPI_GELU) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = gelu_erf(v[i]);
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) fin[i] = v[i];
-  const bool whole = n + 3 < p.N && (p.ld_out & 3) == 0;
-  if constexpr (EPI == EPI_F32) {
-    float *o = p.out_f32 + static_cast<size_t>(t) * p.ld_out + n;
-    if (whole) {
-      *reinterpret_cast<float4 *>(o) = make_float4(v[0], v[1], v[2], v[3]);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (n + i < p.N) o[i] = v[i];
-    }
-  } else if constexpr (EPI == EPI_BF16 || EPI == EPI_GELU) {
-    bf16 *o = p.out_bf16 + static_cast<size_t>(t) * p.ld_out + n;
-    if (whole) {
-      *reinterpret_cast<uint2 *>(o) = pack4_bf16(v);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (n + i < p.N) o[i] = __float2bfloat16(v[i]);
-    }
-  } else if constexpr (EPI == EPI_KV) {
-    // N, q_cols and d_model are multiples of 4 (checked at launch)
-    if (n >= p.N) return;
-    if (n < p.q_cols) {
-      *reinterpret_cast<uint2 *>(p.out_bf16 + static_cast<size_t>(t) * p.ld_out + n) = pack4_bf16(v);
-      return;
-    }
-    const int c = n - p.q_cols;
-    const int which = c / p.d_model;
-    const int hd = c - which * p.d_model;
-    const int2 sp = *tok_local;
-    if (sp.y >= p.ctx) {
-      set_error(p.err, WF_DEV_ERR_CAPACITY);
-      return;
-    }
-    bf16 *dst = which == 0 ? p.kc : p.vc;
-    *reinterpret_cast<uint2 *>(
-        dst + ((static_cast<size_t>(sp.x) * p.n_heads + (hd >> 6)) * p.ctx + sp.y) * 64 + (hd & 63)) =
-        pack4_bf16(v);
-  }
-}
-
-// Epilogue of four consecutive output features n..n+3 of token row t (the
-// staged path).  `old` is the residual row's current value (EPI_RESID).
-// fin[] returns the final values (the updated residual for EPI_RESID) for the
-// LayerNorm statistics.  Four consecutive features never straddle a head or
-// the key/value boundary (multiples of 4), so each store is one vector.
-template <int EPI>
-__device__ __forceinline__ void epi_quad(const GemmParams &p, int t, int n, const float4 &a,
-                                         const float (&b4)[4], const float4 &old,
-                                         const int2 *tok_local, float (&fin)[4]) {
-  float v[4] = {a.x + b4[0], a.y + b4[1], a.z + b4[2], a.w + b4[3]};
-  if constexpr (EPI == EPI_RESID) {
-    // N % 128 == 0 and ld_resid % 4 == 0 (checked at launch): one float4
-    float4 *r = reinterpret_cast<float4 *>(p.resid + static_cast<size_t>(t) * p.ld_resid + n);
-    const float4 nr = make_float4(old.x + v[0], old.y + v[1], old.z + v[2], old.w + v[3]);
-    *r = nr;
-    fin[0] = nr.x;
-    fin[1] = nr.y;
-    fin[2] = nr.z;
-    fin[3] = nr.w;
-    const uint2 h = pack4_bf16(fin);
-    if (p.tap0) *reinterpret_cast<uint2 *>(p.tap0 + static_cast<size_t>(t) * p.ld_tap + n) = h;
-    if (p.tap1) *reinterpret_cast<uint2 *>(p.tap1 + static_cast<size_t>(t) * p.ld_tap + n) = h;
-  } else {
-    epi_quad_out<EPI>(p, t, n, v, tok_local, fin);
   }
 }
 
@@ -1007,6 +913,11 @@ cudaError_t launch_gemm(const void *X, const void *W, GemmParams p, cudaStream_t
   } else if (!X) {
     return cudaErrorInvalidValue;
   }
+  // Past kWideMinM rows pairs of SMs on 256-row weight tiles (same bits).
+  // They write four features at a time whatever the split, so a key/value
+  // scatter with odd strides stays here, as does the output head.
+  const bool quads = p.epi != EPI_KV || !(p.N % 4 || p.q_cols % 4 || p.d_model % 4 || p.ld_out % 4);
+  if (!ln && p.M > kWideMinM && p.epi != EPI_HEAD && quads) return launch_gemm_wide(X, W, p, s, pdl);
   size_t smem = 0;
   if (!plan_gemm(p, &smem)) return cudaErrorInvalidValue;
   const CUtensorMap *tw = tmap_bf16_2d(W, p.N, p.K, kBlockN);

@@ -50,6 +50,7 @@ struct HeadRec {  // one (token row, 128-id vocabulary tile) of the output head
 struct GemmParams {
   int M, N, K;
   int BT, n_tt, splits, kps, stages, pipe_bytes;
+  int n_ptiles;  // gemm_wide: tiles of 256 weight rows by BT tokens
   uint32_t tmem_cols;
   // fold != 0: one CTA computes every split of its tile in turn (the split
   // partials alternate between two TMEM accumulators of acc_cols columns and
@@ -124,6 +125,10 @@ cudaError_t launch_gemm(const void *X, const void *W, GemmParams p, cudaStream_t
 // all of the CTA's token tiles fit in shared memory; otherwise run
 // launch_layernorm first (same bits either way).
 bool gemm_ln_fits(int M, int N, int K, int epi);
+
+// The same projections for many token rows on pairs of SMs (wf_gemm_wide.cu);
+// same arguments and bits as launch_gemm, no LayerNorm-fused operand.
+cudaError_t launch_gemm_wide(const void *X, const void *W, GemmParams p, cudaStream_t s, bool pdl);
 
 // ------------------------------------------------------ skinny projections --
 // Y = X W^T for M <= 16 token rows (wf_skinny.cu): each CTA prefetches its
