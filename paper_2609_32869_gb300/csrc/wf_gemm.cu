@@ -13,16 +13,12 @@
 //
 // K is split into a fixed number of chunks per (N, K) shape so that ~150 CTAs
 // stream weights even for a single sequence.  The S split CTAs of a tile form
-// a thread-block cluster; after the MMAs each stages its fp32 partial tile in
-// its own shared memory and, past a cluster barrier, reduces a slice of the
-// tile by reading the S partials over distributed shared memory in split
-// order, so results are deterministic and independent of M, and no partial
-// ever travels through global memory.  When the token tiles alone give
-// enough CTAs (many sequences), one CTA computes all S splits of its tile in
-// turn ("fold"): the MMA thread alternates the splits between two TMEM
-// accumulators while four warps add each finished partial, in split order,
-// into a third -- the same sums in the same order as the cluster reduction,
-// without its S-fold CTAs, barriers and partial tiles.
+// a thread-block cluster; after the MMAs each pushes its fp32 partials over
+// distributed shared memory to the CTAs that finish the rows, which add them
+// in split order, so results are deterministic and independent of M, and no
+// partial ever travels through global memory.  Past kWideMinM rows the pushes
+// (~16 bytes per cycle and SM) cost more than they save and pairs of SMs run
+// the projection instead (wf_gemm_wide.cu).
 //
 // With programmatic dependent launch the weight tiles of the first pipeline
 // stages are requested before griddepcontrol.wait: they do not depend on the
@@ -47,17 +43,23 @@ constexpr int kStageA = kBlockN * kBlockK * 2;  // 16 KB
 // Shared memory a CTA plans for: two CTAs fit on an SM, so one CTA's
 // epilogue overlaps the other's weight stream.
 constexpr int kSmemBudget = 110 * 1024;
-constexpr int kSmemBudgetAlone = 200 * 1024;  // a CTA that holds all 512 TMEM columns
 constexpr int kSmemBudgetLn = 110 * 1024;  // LN mode: resident token tiles + weight ring
 constexpr int kMaxBT = 128;                // token rows per tile (MMA N)
 constexpr size_t kSmemPerSM = 228 * 1024;  // shared memory of one SM
-constexpr int kLnFuseMaxM = 256;              // token rows up to which LN is fused
-// Token rows above which pairs of SMs take a projection: at 288 rows (32
-// sequences) they halve most launches (fc2 33 -> 17 us, fc1 20 -> 13), while
-// up to 256 rows one token tile covers every row and only split-K over
-// clusters fills the GPU.
-constexpr int kWideMinM = 256;
-constexpr int kFoldMinTiles = 64;             // output tiles from which split-K folds into one CTA
+constexpr uint32_t kGroupBytes = 128 * 4 * 4;  // one split's partials of four token rows
+// Token rows up to which LN is fused: every weight tile normalises the same
+// rows again, which at 144 rows costs 8-15 us per launch against a 4 us
+// LayerNorm kernel; at 32 rows the two forms are within 1%.
+constexpr int kLnFuseMaxM = 64;
+// Token rows above which pairs of SMs (wf_gemm_wide.cu) take a projection from
+// the cluster split-K.  Launches of a captured graph with weights from HBM, us
+// (cluster / pairs): 1280 x 1280 at 64, 96, 144 rows 6.3 / 7.8, 7.2 / 7.8,
+// 8.2 / 7.8; 1280 x 5120 9.8 / 13.9, 12.3 / 13.8, 15.6 / 13.9; 3840 x 1280 (30
+// weight tiles, so the pairs cover the GPU sooner) 7.7 / 7.5, 8.9 / 7.5,
+// 11.9 / 7.9; 5120 x 1280 8.2 / 7.7, 9.7 / 7.9, 12.9 / 8.4.
+constexpr int kWideMinM = 96;
+constexpr int kWideMinMFewRows = 64;
+constexpr int kWideFewRowsN = 3840;
 
 // Epilogue of 16 consecutive token columns t0..t0+15 for output feature n.
 // acc[] holds the 16 accumulated values; every global load of the chunk (the
@@ -202,22 +204,22 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + p.pipe_bytes);
   uint64_t *empty = full + stages;
   uint64_t *done = empty + stages;
-  uint64_t *part_bar = done + 1;  // fold: split partial r finished in accumulator r % 2
-  uint64_t *free_bar = done + 3;  // fold: accumulator r % 2 added into the sum, free again
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 5);
+  uint64_t *inbox_bar = done + 1;  // split-K: the partials of this CTA's token groups arrived
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 2);
   // per-token (slot, position) for EPI_KV, (slot, step) for sampling heads
-  int2 *tok = reinterpret_cast<int2 *>(smem + p.pipe_bytes + (2 * stages + 5) * 8 + 16 + 16);
+  int2 *tok = reinterpret_cast<int2 *>(smem + p.pipe_bytes + (2 * stages + 2) * 8 + 32);
   float2 *lnst = reinterpret_cast<float2 *>(tok + BT);  // per-token (mean, rstd), LN mode
+  // split-K: where the partials of each group of four token rows go (the
+  // cluster addresses of the slot and of its owner's inbox barrier)
+  uint2 *dest = reinterpret_cast<uint2 *>(lnst + (p.ln_x ? BT : 0));
   const bool ln = p.ln_x != nullptr;
   // a bounded wait of this CTA gave up (in the 32 bytes reserved after the
   // barriers, beside the TMEM address; the kernel has no static shared memory)
   volatile int &s_timed_out = *reinterpret_cast<int *>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int tt = blockIdx.x, ntile = blockIdx.y, split = blockIdx.z;
-  const bool fold = p.fold != 0;
-  const int nk = fold ? kps * p.splits : kps;  // k-steps of this CTA
-  const int n0 = ntile * kBlockN, t0 = tt * BT, kit0 = fold ? 0 : split * kps;
+  const int n0 = ntile * kBlockN, t0 = tt * BT, kit0 = split * kps;
 
   if (threadIdx.x == 0) {
     s_timed_out = 0;
@@ -228,13 +230,11 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
       mbar_init(&empty[s], 1);
     }
     mbar_init(done, 1);
-    mbar_init(&part_bar[0], 1);
-    mbar_init(&part_bar[1], 1);
-    mbar_init(&free_bar[0], 4);
-    mbar_init(&free_bar[1], 4);
+    mbar_init(inbox_bar, 1);
     fence_barrier_init();
     fence_proxy_async();
   }
+  __syncwarp();
   if (warp == 2) tmem_alloc(tmem_slot, p.tmem_cols);
   tc_fence_before();
   __syncthreads();
@@ -245,12 +245,16 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   // Weight tiles of the first stages do not depend on the previous kernel:
   // request them before the dependency wait.  In LN mode each stage carries
   // only its weight tile; the token operand is built once for all k-steps.
-  const int npre = nk < stages ? nk : stages;
+  // Copies and MMAs are issued by one elected lane of code that the whole warp
+  // runs: under a lane comparison each of them took ~430 cycles.
+  const int npre = kps < stages ? kps : stages;
   const uint32_t tx = ln ? static_cast<uint32_t>(kStageA) : kStageA + stageB;
-  if (threadIdx.x == 0) {
+  if (warp == 0) {
     for (int i = 0; i < npre; ++i) {
-      mbar_arrive_expect_tx(&full[i], tx);
-      tma_load_2d(sA + static_cast<size_t>(i) * kStageA, &tmW, (kit0 + i) * kBlockK, n0, &full[i]);
+      if (elect_one()) {
+        mbar_arrive_expect_tx(&full[i], tx);
+        tma_load_2d(sA + static_cast<size_t>(i) * kStageA, &tmW, (kit0 + i) * kBlockK, n0, &full[i]);
+      }
     }
   }
   if (ln) {
@@ -260,119 +264,67 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
     __syncthreads();
   }
 
-  int issued = npre;  // k-steps whose tiles the producer (thread 0) has requested
-  if (warp == 0 && lane == 0) {
+  int issued = npre;  // k-steps whose tiles the producer (warp 0) has requested
+  if (warp == 0) {
     // ---------------- TMA producer
     if (!ln) {
       pdl_wait();  // token rows come from the previous kernel
       for (int i = 0; i < npre; ++i)
-        tma_load_2d(sB + static_cast<size_t>(i) * stageB, &tmX, (kit0 + i) * kBlockK, t0, &full[i]);
+        if (elect_one())
+          tma_load_2d(sB + static_cast<size_t>(i) * stageB, &tmX, (kit0 + i) * kBlockK, t0, &full[i]);
     }
-    for (int it = npre; it < nk; ++it) {
-      const int s = it % stages;
-      const uint32_t ph = static_cast<uint32_t>((it / stages) - 1) & 1u;
-      if (!mbar_wait(&empty[s], ph, p.err, p.spin)) {
+    int s = 0;
+    uint32_t ph = 0;
+    for (int it = npre; it < kps; ++it) {  // (only when npre == stages)
+      if (!warp_mbar_wait(&empty[s], ph, p.err, p.spin)) {
         s_timed_out = 1;
         break;
       }
       issued = it + 1;
-      mbar_arrive_expect_tx(&full[s], tx);
-      tma_load_2d(sA + static_cast<size_t>(s) * kStageA, &tmW, (kit0 + it) * kBlockK, n0, &full[s]);
-      if (!ln)
-        tma_load_2d(sB + static_cast<size_t>(s) * stageB, &tmX, (kit0 + it) * kBlockK, t0, &full[s]);
+      if (elect_one()) {
+        mbar_arrive_expect_tx(&full[s], tx);
+        tma_load_2d(sA + static_cast<size_t>(s) * kStageA, &tmW, (kit0 + it) * kBlockK, n0, &full[s]);
+        if (!ln)
+          tma_load_2d(sB + static_cast<size_t>(s) * stageB, &tmX, (kit0 + it) * kBlockK, t0, &full[s]);
+      }
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1;
+      }
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer
-    // Descriptors are built once and stepped: a 16-deep K step is 32 bytes,
-    // +2 in the descriptor's start-address field (shared address >> 4, 14
-    // bits; shared memory is below 256 KB, so the field never carries).  At
-    // small N the single issuing thread, not the tensor pipe, sets the MMA
-    // rate, so the loop keeps everything but the MMAs out of the way.
+  } else if (warp == 1) {
+    // ---------------- MMA issuer.  A 16-deep K step is 32 bytes: +2 in the
+    // descriptors' start-address field (shared address >> 4, 14 bits; shared
+    // memory is below 256 KB, so the field never carries).
     const uint32_t idesc = umma_idesc_bf16(kBlockN, BT);
     const uint64_t a_base = umma_desc_sw128(smem_u32(sA)), b_base = umma_desc_sw128(smem_u32(sB));
-    if (!fold && kps <= stages) {
-      // every k-step has its own stage and none is refilled: wait for all
-      // of them, then issue the MMAs back to back (no per-stage commit)
-      bool landed = true;
-      for (int it = 0; it < kps && landed; ++it) landed = mbar_wait(&full[it], 0u, p.err, p.spin);
-      if (!landed) s_timed_out = 1;
-      if (landed) {
-        tc_fence_after();
-        for (int it = 0; it < kps; ++it) {
-          const uint64_t ad = a_base + static_cast<uint64_t>((it * kStageA) >> 4);
-          const uint64_t bd = b_base + static_cast<uint64_t>((it * stageB) >> 4);
-#pragma unroll
-          for (int kk = 0; kk < kBlockK / 16; ++kk)
-            umma_bf16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (it | kk) != 0 ? 1u : 0u);
-        }
-      }
-    } else {
-      for (int it = 0; it < nk; ++it) {
-        const int s = it % stages;
-        const uint32_t ph = static_cast<uint32_t>(it / stages) & 1u;
-        if (!mbar_wait(&full[s], ph, p.err, p.spin)) {
-          s_timed_out = 1;
-          break;
-        }
-        // fold: split r = it / kps accumulates in columns (r % 2) acc_cols,
-        // once the sum has taken split r - 2 out of them
-        const int r = it / kps, kin = it - r * kps;
-        if (fold && kin == 0 && r >= 2 &&
-            !mbar_wait(&free_bar[r & 1], static_cast<uint32_t>((r >> 1) - 1) & 1u, p.err, p.spin)) {
-          s_timed_out = 1;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t dacc = tmem + (fold ? static_cast<uint32_t>(r & 1) * p.acc_cols : 0u);
-        const uint64_t ad = a_base + static_cast<uint64_t>((s * kStageA) >> 4);
-        const uint64_t bd = b_base + static_cast<uint64_t>(((ln ? it : s) * stageB) >> 4);
-#pragma unroll
-        for (int kk = 0; kk < kBlockK / 16; ++kk)
-          umma_bf16(dacc, ad + 2 * kk, bd + 2 * kk, idesc, (kin | kk) != 0 ? 1u : 0u);
-        umma_commit(&empty[s]);
-        if (fold && kin == kps - 1) umma_commit(&part_bar[r & 1]);
-      }
-    }
-    umma_commit(done);
-  }
-  __syncwarp();
-
-  // ---------------- fold: warps 4..7 (TMEM lane quarters 0..3) add each split
-  // partial into the sum columns 2 acc_cols.., in split order from zero
-  if (fold && warp >= 4) {
-    const uint32_t lbase = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-    const uint32_t sum_col = lbase + 2 * p.acc_cols;
-    const int n_ch = BT / 16;
-    for (int r = 0; r < p.splits; ++r) {
-      if (!mbar_wait(&part_bar[r & 1], static_cast<uint32_t>(r >> 1) & 1u, p.err, p.spin)) {
+    int s = 0;
+    uint32_t ph = 0;
+    for (int it = 0; it < kps; ++it) {
+      if (!warp_mbar_wait(&full[s], ph, p.err, p.spin)) {
         s_timed_out = 1;
         break;
       }
       tc_fence_after();
-      const uint32_t part_col = lbase + static_cast<uint32_t>(r & 1) * p.acc_cols;
-      for (int c = 0; c < n_ch; ++c) {
-        float v[16], a[16];
-        tmem_ld16(part_col + c * 16, v);
-        if (r == 0) {
+      if (elect_one()) {
+        const uint64_t ad = a_base + static_cast<uint64_t>((s * kStageA) >> 4);
+        const uint64_t bd = b_base + static_cast<uint64_t>(((ln ? it : s) * stageB) >> 4);
 #pragma unroll
-          for (int e = 0; e < 16; ++e) a[e] = 0.f + v[e];
-        } else {
-          tmem_ld16(sum_col + c * 16, a);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) a[e] += v[e];
-        }
-        tmem_st16(sum_col + c * 16, a);
+        for (int kk = 0; kk < kBlockK / 16; ++kk)
+          umma_bf16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (it | kk) != 0 ? 1u : 0u);
+        umma_commit(&empty[s]);
       }
-      tmem_st_wait();
-      tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cta(&free_bar[r & 1]);
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1;
+      }
     }
+    if (elect_one()) umma_commit(done);
   }
+  __syncwarp();
 
   // ---------------- epilogue: warp w owns TMEM lanes [32w, 32w+32) = weight rows
-  // (fold: the sum columns; S_eff = 1, the CTA finishes every row of its tile)
-  const int S_eff = fold ? 1 : p.splits;
   pdl_wait();
   if constexpr (EPI == EPI_HEAD) {
     if (p.temperature > 0.f) {
@@ -404,26 +356,42 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   // result load while the MMAs run: the bias of the lane's four features and,
   // for a residual update, the first row this warp will own.
   const int cols = max(0, min(BT, p.M - t0));
+  // split-K: the tile's groups of four token rows, and those this CTA finishes
+  const int S = p.splits, n_grp = (cols + 3) / 4;
+  const int g_lo = n_grp * split / S, g_hi = n_grp * (split + 1) / S;
+  if (EPI != EPI_HEAD && S > 1) {
+    const int g_max = (n_grp + S - 1) / S;
+    if (threadIdx.x == 0)
+      mbar_arrive_expect_tx(inbox_bar, static_cast<uint32_t>(S * (g_hi - g_lo)) * kGroupBytes);
+    for (int g = threadIdx.x; g < n_grp; g += kThreads) {
+      const int owner = ((g + 1) * S - 1) / n_grp, lg = g - n_grp * owner / S;
+      dest[g] = make_uint2(dsmem_map(smem_u32(smem) + static_cast<uint32_t>(split * g_max + lg) * kGroupBytes, owner),
+                           dsmem_map(smem_u32(inbox_bar), owner));
+    }
+  }
   float b4[4] = {0.f, 0.f, 0.f, 0.f};
-  float4 pre = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool has_pre = false;
-  if (EPI != EPI_HEAD && (S_eff > 1 || p.stats_out)) {
+  // (split-K: a warp's first group of four rows)
+  float4 pre[4];
+  if (EPI != EPI_HEAD && (S > 1 || p.stats_out)) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int nn = n0 + 4 * lane + i;
       b4[i] = (p.bias && nn < p.N) ? bf2f(p.bias[nn]) : 0.f;
     }
-    if constexpr (EPI == EPI_RESID) {
-      const int S = S_eff, tl = cols * split / S + warp;
-      if (tl < cols * (split + 1) / S) {
-        pre = *reinterpret_cast<const float4 *>(p.resid + static_cast<size_t>(t0 + tl) * p.ld_resid +
-                                                n0 + 4 * lane);
-        has_pre = true;
-      }
-    }
   }
+  auto load_group = [&](int g) {  // the residual rows of group g
+    if constexpr (EPI == EPI_RESID) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        pre[k] = 4 * g + k < cols
+                     ? *reinterpret_cast<const float4 *>(p.resid + static_cast<size_t>(t0 + 4 * g + k) * p.ld_resid +
+                                                         n0 + 4 * lane)
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  if (S > 1 && g_lo + warp < g_hi) load_group(g_lo + warp);
   __syncthreads();
-  const bool ok = mbar_wait(done, 0, p.err, p.spin);
+  bool ok = mbar_wait(done, 0, p.err, p.spin);
   if (!ok) s_timed_out = 1;
   tc_fence_after();
   __syncwarp();
@@ -431,8 +399,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   // token-column chunks [c_lo, c_hi) of its half of the tile
   const int quarter = warp & 3, half = warp >> 2;
   const int n = n0 + quarter * 32 + lane;
-  const uint32_t trow =
-      tmem + (static_cast<uint32_t>(quarter * 32) << 16) + (fold ? 2 * p.acc_cols : 0u);
+  const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
   const int n_chunks = BT / 16, c_per = (n_chunks + 1) / 2;
   const int c_lo = half * c_per, c_hi = min(n_chunks, c_lo + c_per);
 
@@ -494,7 +461,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
         p.recs[static_cast<size_t>(t) * n_tiles + ntile] = rec;
       }
     }
-  } else if (S_eff == 1 && !p.stats_out) {
+  } else if (p.splits == 1 && !p.stats_out) {
     const float bn = (p.bias && n < p.N) ? bf2f(p.bias[n]) : 0.f;
     for (int c = c_lo; c < c_hi; ++c) {
       float v[16];
@@ -502,25 +469,10 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
       if (ok) epi_chunk<EPI>(p, t0 + c * 16, n, bn, v, tok + c * 16);
     }
   } else {
-    // Four-feature epilogue: a warp owns a token row (lane l: features
-    // 4l..4l+3), so the row's LayerNorm statistics over this 128-feature tile
-    // are two warp reductions.  Split-K partials are summed in split order.
-    const int S = S_eff;
-    const int rank = fold ? 0 : split;  // cluster (1, 1, S) over gridDim.z == S: rank == blockIdx.z
-    const int rlo = cols * rank / S, rhi = cols * (rank + 1) / S;
+    // Four-feature epilogue: a warp owns token rows (lane l: features
+    // 4l..4l+3), so a row's LayerNorm statistics over this 128-feature tile
+    // are two warp reductions.
     const int stat_tiles = p.N / kBlockN;
-    // the residual row a warp updates next (EPI_RESID; the first one was
-    // loaded under the MMAs)
-    auto load_old = [&](int tl) {
-      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-      if constexpr (EPI == EPI_RESID) {
-        o = (has_pre && tl == rlo + warp)
-                ? pre
-                : *reinterpret_cast<const float4 *>(p.resid + static_cast<size_t>(t0 + tl) * p.ld_resid +
-                                                    n0 + 4 * lane);
-      }
-      return o;
-    };
     auto finish_row = [&](int tl, const float4 &acc, bool valid, const float4 &old) {
       float fin[4] = {0.f, 0.f, 0.f, 0.f};
       if (valid) epi_quad<EPI>(p, t0 + tl, n0 + 4 * lane, acc, b4, old, tok + tl, fin);
@@ -533,69 +485,79 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
       }
     };
     const int r = quarter * 32 + lane;
-    // Every CTA stages its fp32 tile [BT][128] in its own shared memory (the
-    // pipeline buffers are free once the MMAs completed); with split-K the S
-    // CTAs of the tile form a cluster and each reduces its share of the token
-    // rows by reading the S partials over DSMEM.
     float *tile = reinterpret_cast<float *>(smem);
-    for (int c = c_lo; c < c_hi; ++c) {
-      float v[16];
-      tmem_ld16(trow + c * 16, v);
+    if (S > 1) {
+      // Split-K: every CTA pushes its fp32 partials of each group of four
+      // token rows into the inbox of the CTA that finishes the group (over the
+      // pipeline buffers, free once all CTAs' MMAs are done), 16 bytes (four
+      // tokens of one feature) per asynchronous store; the inbox's barrier
+      // counts the bytes.  The owner adds the S partials in split order from
+      // its own shared memory.  From the last MMA to the CTA's end this takes
+      // 1400 cycles at 9 rows and 4200 at 64 (1280 x 1280); pulling over DSMEM
+      // between two release / acquire cluster barriers took 4300 and 6000.
+      cluster_arrive_relaxed();
+      cluster_wait();
+      const int pos = (r & ~3) | ((r + (r >> 3)) & 3);  // conflict-free for the owner's reads
+      for (int c = c_lo; c < c_hi; ++c) {
+        float v[16];
+        tmem_ld16_issue(trow + c * 16, v);
+        tmem_ld_wait(v);
 #pragma unroll
-      for (int jj = 0; jj < 16; ++jj) tile[(c * 16 + jj) * kBlockN + r] = v[jj];
-    }
-    if (S > 1) cluster_sync();
-    else __syncthreads();
-    const uint32_t tile_u32 = smem_u32(tile);
-    auto reduce_row = [&](int tl) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      const int e = tl * kBlockN + 4 * lane;
-      if (S == 1) {
-        acc = *reinterpret_cast<const float4 *>(tile + e);
-      } else {
+        for (int k = 0; k < 4; ++k) {
+          const int g = c * 4 + k;
+          if (g >= n_grp) break;
+          const uint2 d = dest[g];
+          dsmem_push_f32x4(d.x + 16u * pos, make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]), d.y);
+        }
+      }
+      if (!mbar_wait(inbox_bar, 0, p.err, p.spin)) {
+        ok = false;
+        s_timed_out = 1;
+        // partials on their way into this CTA must land before it leaves
+        mbar_drain(inbox_bar, 0);
+      }
+      __syncwarp();
+      const int g_max = (n_grp + S - 1) / S;
+      for (int g = g_lo + warp; g < g_hi; g += kThreads / 32) {
+        if (g != g_lo + warp) load_group(g);
+        const float4 *in = reinterpret_cast<const float4 *>(smem + static_cast<size_t>(g - g_lo) * kGroupBytes);
+        float4 acc[4];  // feature 4 lane + i, its four tokens
 #pragma unroll
-        for (int sp = 0; sp < 16; ++sp) {
-          if (sp < S) {
-            const float4 v = dsmem_ld_f32x4(dsmem_map(tile_u32 + 4u * e, sp));
-            acc.x += v.x;
-            acc.y += v.y;
-            acc.z += v.z;
-            acc.w += v.w;
+        for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int sp = 0; sp < S; ++sp) {
+          const float4 *src = in + static_cast<size_t>(sp * g_max) * (kGroupBytes / 16);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 v = src[4 * lane + ((i + (lane >> 1)) & 3)];
+            acc[i].x += v.x;
+            acc[i].y += v.y;
+            acc[i].z += v.z;
+            acc[i].w += v.w;
           }
         }
-      }
-      return acc;
-    };
-    constexpr int W = kThreads / 32;
-    if (S > 1 && rhi - rlo <= 2 * W) {
-      // at most two rows per warp: read every partial first, tell the peers
-      // their tiles are free, then run the epilogue while they finish
-      float4 acc[2], old[2];
+        const float4 row[4] = {make_float4(acc[0].x, acc[1].x, acc[2].x, acc[3].x),
+                               make_float4(acc[0].y, acc[1].y, acc[2].y, acc[3].y),
+                               make_float4(acc[0].z, acc[1].z, acc[2].z, acc[3].z),
+                               make_float4(acc[0].w, acc[1].w, acc[2].w, acc[3].w)};
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        if (rlo + warp + W * k < rhi) {
-          old[k] = load_old(rlo + warp + W * k);
-          acc[k] = reduce_row(rlo + warp + W * k);
-        }
+        for (int k = 0; k < 4; ++k)
+          if (4 * g + k < cols) finish_row(4 * g + k, row[k], ok, pre[k]);
       }
-      cluster_arrive();
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-        if (rlo + warp + W * k < rhi) finish_row(rlo + warp + W * k, acc[k], ok, old[k]);
-      cluster_wait();
     } else {
-      // two rows per warp at a time, so their loads overlap
-      for (int tl = rlo + warp; tl < rhi; tl += 2 * W) {
-        const int tl2 = tl + W;
-        const bool two = tl2 < rhi;
-        const float4 old1 = load_old(tl);
-        const float4 old2 = two ? load_old(tl2) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 acc1 = reduce_row(tl);
-        const float4 acc2 = two ? reduce_row(tl2) : make_float4(0.f, 0.f, 0.f, 0.f);
-        finish_row(tl, acc1, ok, old1);
-        if (two) finish_row(tl2, acc2, ok, old2);
+      for (int c = c_lo; c < c_hi; ++c) {
+        float v[16];
+        tmem_ld16(trow + c * 16, v);
+#pragma unroll
+        for (int jj = 0; jj < 16; ++jj) tile[(c * 16 + jj) * kBlockN + r] = v[jj];
       }
-      if (S > 1) cluster_sync();
+      __syncthreads();
+      for (int tl = warp; tl < cols; tl += kThreads / 32) {
+        float4 old = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (EPI == EPI_RESID)
+          old = *reinterpret_cast<const float4 *>(p.resid + static_cast<size_t>(t0 + tl) * p.ld_resid + n0 + 4 * lane);
+        finish_row(tl, *reinterpret_cast<const float4 *>(tile + tl * kBlockN + 4 * lane), ok, old);
+      }
     }
   }
 
@@ -753,7 +715,7 @@ static cudaError_t cluster_fits(int splits, size_t smem, dim3 grid) {
 template <int EPI>
 static cudaError_t launch_typed(const CUtensorMap *tw, const CUtensorMap *tx, const GemmParams &p,
                                 size_t smem, cudaStream_t s, bool pdl) {
-  const bool clustered = p.splits > 1 && !p.fold;
+  const bool clustered = p.splits > 1;
   const dim3 grid(p.n_tt, (p.N + kBlockN - 1) / kBlockN, clustered ? p.splits : 1);
   if (clustered) {
     cudaError_t e = cluster_fits<EPI>(p.splits, smem, grid);
@@ -825,24 +787,14 @@ static bool plan_gemm(GemmParams &p, size_t *smem_out) {
   if (k_iters % p.splits) return false;
   p.kps = k_iters / p.splits;
   const bool ln = p.ln_x != nullptr;
-  // fold the splits into one CTA when the token tiles alone fill the GPU
-  const int n_tiles = (p.N + kBlockN - 1) / kBlockN;
-  p.fold = (!ln && p.epi != EPI_HEAD && p.splits > 1 && p.n_tt * n_tiles >= kFoldMinTiles) ? 1 : 0;
   const size_t stageA = kStageA, stageB = static_cast<size_t>(p.BT) * kBlockK * 2;
-  const size_t red = static_cast<size_t>(p.BT) * sizeof(int2) * (ln ? 2 : 1);
+  const size_t red = static_cast<size_t>(p.BT) * sizeof(int2) * (ln ? 2 : 1) +
+                     (p.splits > 1 ? static_cast<size_t>(p.BT / 4) * sizeof(uint2) : 0);
   const size_t fixed = red;
   uint32_t cols = 32;
   while (cols < static_cast<uint32_t>(p.BT)) cols <<= 1;
-  p.acc_cols = cols;
-  if (p.fold) {  // two split accumulators and their sum
-    uint32_t all = 32;
-    while (all < 3 * cols) all <<= 1;
-    if (all > 512) return false;
-    cols = all;
-  }
   p.tmem_cols = cols;
-  // a CTA that holds all of TMEM is alone on its SM: it may take a deeper ring
-  const size_t budget = cols == 512 ? kSmemBudgetAlone : kSmemBudget;
+  const size_t budget = kSmemBudget;
   int stages;
   size_t pipe;
   if (ln) {
@@ -856,16 +808,16 @@ static bool plan_gemm(GemmParams &p, size_t *smem_out) {
   } else {
     if (fixed + stageA + stageB > budget) return false;
     stages = static_cast<int>((budget - fixed) / (stageA + stageB));
-    const int nk = p.fold ? p.kps * p.splits : p.kps;
-    if (stages > nk) stages = nk;
+    if (stages > p.kps) stages = p.kps;
     if (stages > 16) stages = 16;
     pipe = stages * (stageA + stageB);
   }
   p.stages = stages;
   // the staged epilogues reuse the pipeline buffers for a [BT][128] fp32 tile
-  if ((p.splits > 1 && !p.fold) || p.stats_out || p.epi == EPI_HEAD)
-    pipe = std::max<size_t>(pipe, 512 * static_cast<size_t>(p.BT));
-  size_t smem = 1024 + pipe + (2 * stages + 5) * 8 + 32 + 16 + red;
+  if (p.stats_out || p.epi == EPI_HEAD) pipe = std::max<size_t>(pipe, 512 * static_cast<size_t>(p.BT));
+  if (p.splits > 1)  // inbox: every split's partials of the CTA's share of the token groups
+    pipe = std::max<size_t>(pipe, static_cast<size_t>(p.splits) * ((p.BT / 4 + p.splits - 1) / p.splits) * kGroupBytes);
+  size_t smem = 1024 + pipe + (2 * stages + 2) * 8 + 32 + 16 + red;
   // A CTA blocks in tcgen05.alloc while co-resident CTAs hold the SM's 512
   // TMEM columns; CTAs of one cluster wait for each other, so no more CTAs
   // may fit on an SM (by shared memory) than can hold TMEM at once.
@@ -917,7 +869,8 @@ cudaError_t launch_gemm(const void *X, const void *W, GemmParams p, cudaStream_t
   // They write four features at a time whatever the split, so a key/value
   // scatter with odd strides stays here, as does the output head.
   const bool quads = p.epi != EPI_KV || !(p.N % 4 || p.q_cols % 4 || p.d_model % 4 || p.ld_out % 4);
-  if (!ln && p.M > kWideMinM && p.epi != EPI_HEAD && quads) return launch_gemm_wide(X, W, p, s, pdl);
+  const int wide_m = p.N >= kWideFewRowsN ? kWideMinMFewRows : kWideMinM;
+  if (!ln && p.M > wide_m && p.epi != EPI_HEAD && quads) return launch_gemm_wide(X, W, p, s, pdl);
   size_t smem = 0;
   if (!plan_gemm(p, &smem)) return cudaErrorInvalidValue;
   const CUtensorMap *tw = tmap_bf16_2d(W, p.N, p.K, kBlockN);

@@ -12,8 +12,10 @@
 // accumulators: eight epilogue warps work on one while the MMAs fill the
 // other.
 //
-// What bounds it: at 864 rows the operand fetch through L2 and the issuing
-// warps' ~300 cycles per 64-column k-step (barrier wait, issue, commit).
+// What bounds it: the copies' rate, ~85 bytes per cycle and SM (a 64-column
+// k-step of 128 weight rows and 16 token rows takes ~220 cycles whatever the
+// MMAs do; prefetching the weights into L2 first takes the same engine and
+// measured 5-15% slower).
 // Measured against wf_gemm.cu's folded split-K at 864 rows (one launch, cold):
 // out / cross out / fc2 36 -> 15 us on average, fc1 39 -> 23, QKV 37 -> 19,
 // cross query 18 -> 11; acoustic K/V of 8 requests (12000 x 2560 x 1280)
@@ -43,7 +45,7 @@ constexpr int kWideThreads = 384;
 constexpr int kWideEpiWarp = 4;      // first epilogue warp
 constexpr int kWideBK = 64;               // K per stage (one 128-byte swizzle atom)
 constexpr int kWideA = 128 * kWideBK * 2;  // weight tile: [128 rows][128 B]
-constexpr int kWideMaxStages = 8;
+constexpr int kWideMaxStages = 10;
 constexpr int kWideSlice = 16;       // token rows per staging buffer
 constexpr int kWideStage = 4 * kWideSlice * 128 * 4;  // two buffers per half of the columns
 constexpr int kWideAcc = 256;        // TMEM columns per accumulator
@@ -54,11 +56,6 @@ constexpr int kWideBars = (2 * kWideMaxStages + 5) * 8;
 constexpr int kWideTok = 2 * 256 * 8;  // (slot, position) per token row, two tiles
 constexpr int kWideFixed = 1024 + kWideStage + kWideTok + kWideBars + 32;
 
-// mbar_wait by a converged warp: every lane waits, one answer.
-__device__ __forceinline__ bool warp_mbar_wait(uint64_t *bar, uint32_t parity, uint32_t *err, long long limit) {
-  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, limit));
-}
 __device__ __forceinline__ void half_barrier(int hg) {  // the four epilogue warps of a column half
   asm volatile("bar.sync %0, 128;" ::"r"(1 + hg) : "memory");
 }

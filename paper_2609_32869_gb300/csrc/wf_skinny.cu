@@ -85,9 +85,6 @@ __device__ __forceinline__ uint32_t a_off(int M, int r, int k) {
   return static_cast<uint32_t>(line * 128 + ((((k >> 3) & 7) ^ (line & 7)) << 4) + (k & 7) * 2);
 }
 
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void dsmem_st_f32(uint32_t cluster_addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
 }
