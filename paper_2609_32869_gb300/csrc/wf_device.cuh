@@ -287,6 +287,24 @@ __device__ __forceinline__ void tmem_ld_wait(float *v) {
                :
                : "memory");
 }
+// C (8 or 16) columns, complete on return.
+template <int C>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float *v) {
+  static_assert(C == 8 || C == 16, "columns per load");
+  if constexpr (C == 16) {
+    tmem_ld16_issue(taddr, v);
+    tmem_ld_wait(v);
+  } else {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "r"(taddr)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])
+                 :
+                 : "memory");
+  }
+}
 
 // ---------------------------------------------------------- clusters ----
 __device__ __forceinline__ void cluster_sync() {
@@ -417,6 +435,16 @@ __device__ __forceinline__ float ln_apply(float x, float2 ms, float g, float b) 
 }
 
 // ---------------------------------------------------------- numerics ----
+__device__ __forceinline__ float lg2f_fast(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float exp2f_fast(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ float bf2f(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ float gelu_erf(float x) {
   return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f));

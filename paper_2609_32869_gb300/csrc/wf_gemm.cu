@@ -326,20 +326,6 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
 
   // ---------------- epilogue: warp w owns TMEM lanes [32w, 32w+32) = weight rows
   pdl_wait();
-  if constexpr (EPI == EPI_HEAD) {
-    if (p.temperature > 0.f) {
-      for (int j = threadIdx.x; j < BT; j += blockDim.x) {
-        const int t = t0 + j;
-        int2 ss = make_int2(0, 0);
-        if (t < p.M) {
-          const int i = t / p.rows_per_seq;
-          ss.x = p.seq_slot[i];
-          ss.y = p.step[ss.x];
-        }
-        tok[j] = ss;
-      }
-    }
-  }
   if constexpr (EPI == EPI_KV) {
     for (int j = threadIdx.x; j < BT; j += blockDim.x) {
       const int t = t0 + j;
@@ -359,7 +345,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   // split-K: the tile's groups of four token rows, and those this CTA finishes
   const int S = p.splits, n_grp = (cols + 3) / 4;
   const int g_lo = n_grp * split / S, g_hi = n_grp * (split + 1) / S;
-  if (EPI != EPI_HEAD && S > 1) {
+  if (S > 1) {
     const int g_max = (n_grp + S - 1) / S;
     if (threadIdx.x == 0)
       mbar_arrive_expect_tx(inbox_bar, static_cast<uint32_t>(S * (g_hi - g_lo)) * kGroupBytes);
@@ -372,7 +358,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   float b4[4] = {0.f, 0.f, 0.f, 0.f};
   // (split-K: a warp's first group of four rows)
   float4 pre[4];
-  if (EPI != EPI_HEAD && (S > 1 || p.stats_out)) {
+  if (S > 1 || p.stats_out) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int nn = n0 + 4 * lane + i;
@@ -403,65 +389,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   const int n_chunks = BT / 16, c_per = (n_chunks + 1) / 2;
   const int c_lo = half * c_per, c_hi = min(n_chunks, c_lo + c_per);
 
-  if constexpr (EPI == EPI_HEAD) {
-    // Stage the [BT][128] logit tile in shared memory (the pipeline buffers
-    // are free once the MMAs completed); then a warp owns a token row, lane l
-    // folds features 4l..4l+3 in order and the warp combines its lanes:
-    // running max with the lowest id on ties, sum of exp(x - max), and the
-    // Gumbel-max draw.  One record per (row, vocabulary tile).
-    const bool sampling = p.temperature > 0.f;
-    const int n_tiles = gridDim.y;
-    float *tile = reinterpret_cast<float *>(smem);
-    const int r = quarter * 32 + lane;
-    for (int c = c_lo; c < c_hi; ++c) {
-      float v[16];
-      tmem_ld16(trow + c * 16, v);
-#pragma unroll
-      for (int jj = 0; jj < 16; ++jj) tile[(c * 16 + jj) * kBlockN + r] = v[jj];
-    }
-    __syncthreads();
-    constexpr int W = kThreads / 32;
-    for (int tl = warp; tl < cols; tl += W) {
-      const int t = t0 + tl;
-      const float4 z4 = *reinterpret_cast<const float4 *>(tile + tl * kBlockN + 4 * lane);
-      const float z[4] = {z4.x, z4.y, z4.z, z4.w};
-      const int2 ss = sampling ? tok[tl] : make_int2(0, 0);
-      const int j = t % p.rows_per_seq;
-      float m = -INFINITY, sum = 0.f, gm = -INFINITY;
-      int arg = 0x7fffffff, garg = 0x7fffffff;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int nn = n0 + 4 * lane + i;
-        const bool masked = nn >= p.N || (p.suppress && p.suppress[nn]);
-        if (ok && p.logits && nn < p.N) p.logits[static_cast<size_t>(t) * p.N + nn] = z[i];
-        const float x = masked ? -INFINITY : (sampling ? __fdiv_rn(z[i], p.temperature) : z[i]);
-        float g = -INFINITY;
-        if (sampling && !masked)
-          g = x + gumbel(p.seed, static_cast<uint32_t>(ss.x), static_cast<uint32_t>(ss.y),
-                         static_cast<uint32_t>(j), p.tag, static_cast<uint32_t>(nn));
-        head_combine(m, sum, arg, gm, garg, x, masked ? 0.f : 1.f, nn, g, nn);
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float m2 = __shfl_down_sync(0xffffffffu, m, off);
-        const float s2 = __shfl_down_sync(0xffffffffu, sum, off);
-        const float gm2 = __shfl_down_sync(0xffffffffu, gm, off);
-        const int a2 = __shfl_down_sync(0xffffffffu, arg, off);
-        const int ga2 = __shfl_down_sync(0xffffffffu, garg, off);
-        head_combine(m, sum, arg, gm, garg, m2, s2, a2, gm2, ga2);
-      }
-      if (lane == 0 && ok) {
-        HeadRec rec;
-        rec.m = m;
-        rec.s = sum;
-        rec.gm = gm;
-        rec.arg = arg;
-        rec.garg = garg;
-        rec._pad[0] = rec._pad[1] = rec._pad[2] = 0;
-        p.recs[static_cast<size_t>(t) * n_tiles + ntile] = rec;
-      }
-    }
-  } else if (p.splits == 1 && !p.stats_out) {
+  if (p.splits == 1 && !p.stats_out) {
     const float bn = (p.bias && n < p.N) ? bf2f(p.bias[n]) : 0.f;
     for (int c = c_lo; c < c_hi; ++c) {
       float v[16];
@@ -759,8 +687,6 @@ cudaError_t gemm_init() {
       status = cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     if (status == cudaSuccess)
       status = cudaFuncSetAttribute(gemm_tc_kernel<EPI_KV>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if (status == cudaSuccess)
-      status = cudaFuncSetAttribute(gemm_tc_kernel<EPI_HEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     // split-K clusters of up to 16 CTAs
     const void *fns[] = {reinterpret_cast<const void *>(gemm_tc_kernel<EPI_F32>),
                          reinterpret_cast<const void *>(gemm_tc_kernel<EPI_BF16>),
@@ -772,7 +698,6 @@ cudaError_t gemm_init() {
         status = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     for (const void *f : fns)
       if (status == cudaSuccess) status = prefer_max_shared(f);
-    if (status == cudaSuccess) status = prefer_max_shared(reinterpret_cast<const void *>(gemm_tc_kernel<EPI_HEAD>));
   });
   return status;
 }
@@ -781,7 +706,6 @@ cudaError_t gemm_init() {
 static bool plan_gemm(GemmParams &p, size_t *smem_out) {
   if (p.M <= 0 || p.N <= 0 || p.K <= 0 || p.K % kBlockK) return false;
   gemm_token_tiling(p.M, &p.BT, &p.n_tt);
-  if (p.epi == EPI_HEAD) p.splits = 1;
   if (p.splits < 1) p.splits = 1;
   const int k_iters = p.K / kBlockK;
   if (k_iters % p.splits) return false;
@@ -814,7 +738,7 @@ static bool plan_gemm(GemmParams &p, size_t *smem_out) {
   }
   p.stages = stages;
   // the staged epilogues reuse the pipeline buffers for a [BT][128] fp32 tile
-  if (p.stats_out || p.epi == EPI_HEAD) pipe = std::max<size_t>(pipe, 512 * static_cast<size_t>(p.BT));
+  if (p.stats_out) pipe = std::max<size_t>(pipe, 512 * static_cast<size_t>(p.BT));
   if (p.splits > 1)  // inbox: every split's partials of the CTA's share of the token groups
     pipe = std::max<size_t>(pipe, static_cast<size_t>(p.splits) * ((p.BT / 4 + p.splits - 1) / p.splits) * kGroupBytes);
   size_t smem = 1024 + pipe + (2 * stages + 2) * 8 + 32 + 16 + red;
@@ -867,10 +791,11 @@ cudaError_t launch_gemm(const void *X, const void *W, GemmParams p, cudaStream_t
   }
   // Past kWideMinM rows pairs of SMs on 256-row weight tiles (same bits).
   // They write four features at a time whatever the split, so a key/value
-  // scatter with odd strides stays here, as does the output head.
+  // scatter with odd strides stays here.  They run the output head at any
+  // number of rows.
   const bool quads = p.epi != EPI_KV || !(p.N % 4 || p.q_cols % 4 || p.d_model % 4 || p.ld_out % 4);
   const int wide_m = p.N >= kWideFewRowsN ? kWideMinMFewRows : kWideMinM;
-  if (!ln && p.M > wide_m && p.epi != EPI_HEAD && quads) return launch_gemm_wide(X, W, p, s, pdl);
+  if (p.epi == EPI_HEAD || (!ln && p.M > wide_m && quads)) return launch_gemm_wide(X, W, p, s, pdl);
   size_t smem = 0;
   if (!plan_gemm(p, &smem)) return cudaErrorInvalidValue;
   const CUtensorMap *tw = tmap_bf16_2d(W, p.N, p.K, kBlockN);
@@ -882,7 +807,6 @@ cudaError_t launch_gemm(const void *X, const void *W, GemmParams p, cudaStream_t
     case EPI_GELU: return launch_typed<EPI_GELU>(tw, tx, p, smem, s, pdl);
     case EPI_RESID: return launch_typed<EPI_RESID>(tw, tx, p, smem, s, pdl);
     case EPI_KV: return launch_typed<EPI_KV>(tw, tx, p, smem, s, pdl);
-    case EPI_HEAD: return launch_typed<EPI_HEAD>(tw, tx, p, smem, s, pdl);
     default: return cudaErrorInvalidValue;
   }
 }

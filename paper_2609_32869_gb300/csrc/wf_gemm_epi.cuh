@@ -1,26 +1,10 @@
 // Epilogue arithmetic shared by the tcgen05 projection kernels: four output
-// features of one token row at a time, and the output head's record combine.
+// features of one token row at a time.
 #pragma once
 #include "wf_device.cuh"
 #include "wf_internal.h"
 
 namespace wf {
-
-__device__ __forceinline__ void head_combine(float &m, float &s, int &arg, float &gm, int &garg,
-                                             float m2, float s2, int arg2, float gm2, int garg2) {
-  const float M = fmaxf(m, m2);
-  float ns = 0.f;
-  if (M != -INFINITY) {
-    ns = (m == -INFINITY ? 0.f : s * __expf(m - M)) + (m2 == -INFINITY ? 0.f : s2 * __expf(m2 - M));
-  }
-  if (m2 > m || (m2 == m && arg2 < arg)) arg = arg2;
-  m = M;
-  s = ns;
-  if (gm2 > gm || (gm2 == gm && garg2 < garg)) {
-    gm = gm2;
-    garg = garg2;
-  }
-}
 
 // Four floats as four bf16 (round to nearest even) in one 8-byte word.
 __device__ __forceinline__ uint2 pack4_bf16(const float (&v)[4]) {

@@ -23,16 +23,21 @@
 // columns instead of 64 (fewer barrier rounds, a shallower ring) measured 10%
 // slower there, and every single token tile of 64, 96 or 128 rows 2-5% slower
 // over a 96-sequence step than the choice of gemm_wide_plan.
+// The output head (51866 x 1280) runs here at any number of rows: against one
+// CTA per 128 ids and token tile, whose epilogue folded (max, sum, argmax,
+// Gumbel) records through five shuffles per step, 33 -> 28 us at 9 rows (one
+// read of the weights is 20), 61 -> 30 at 144, 304 -> 86 at 864, and sampling
+// 288 rows 205 -> 86.
 //
 // Arithmetic: K is cut into the same `splits` chunks as the cluster split-K of
 // wf_gemm.cu, each chunk accumulates on its own in TMEM, and the chunks are
 // added in order from zero in fp32 (in registers), so a row's bits do not
 // depend on which of the two kernels ran it.
 //
-// Roles per CTA (384 threads): warp 0 requests its CTA's tiles by TMA; warp 1
-// of the even CTA issues the MMAs; warp 2 owns TMEM; warps 4..11 run the
-// epilogue, two per TMEM lane quarter (low and high half of the token
-// columns).
+// Roles per CTA: warp 0 requests its CTA's tiles by TMA; warp 1
+// of the even CTA issues the MMAs; warp 2 owns TMEM; warps 4 and on run the
+// epilogue, two or four per TMEM lane quarter, each with its group of the
+// token columns.
 #include <mutex>
 
 #include "wf_device.cuh"
@@ -41,13 +46,19 @@
 
 namespace wf {
 
-constexpr int kWideThreads = 384;
 constexpr int kWideEpiWarp = 4;      // first epilogue warp
 constexpr int kWideBK = 64;               // K per stage (one 128-byte swizzle atom)
 constexpr int kWideA = 128 * kWideBK * 2;  // weight tile: [128 rows][128 B]
 constexpr int kWideMaxStages = 10;
-constexpr int kWideSlice = 16;       // token rows per staging buffer
-constexpr int kWideStage = 4 * kWideSlice * 128 * 4;  // two buffers per half of the columns
+constexpr int kWideStage = 64 * 128 * 4;  // two staging buffers per column group, 64 token rows in all
+// Epilogue warps: two per TMEM lane quarter, four for the output head, whose
+// per-id arithmetic needs the latency hiding (51866 ids, one launch, cold:
+// sampling 288 rows 116 us with eight warps, 86 with sixteen; greedy 864 rows
+// with their logits 116 and 86).
+template <int EPI>
+constexpr int kWideEpiWarps = EPI == EPI_HEAD ? 16 : 8;
+template <int EPI>
+constexpr int kWideThreads = 32 * (4 + kWideEpiWarps<EPI>);
 constexpr int kWideAcc = 256;        // TMEM columns per accumulator
 constexpr uint32_t kWideTmem = 512;
 
@@ -56,16 +67,169 @@ constexpr int kWideBars = (2 * kWideMaxStages + 5) * 8;
 constexpr int kWideTok = 2 * 256 * 8;  // (slot, position) per token row, two tiles
 constexpr int kWideFixed = 1024 + kWideStage + kWideTok + kWideBars + 32;
 
-__device__ __forceinline__ void half_barrier(int hg) {  // the four epilogue warps of a column half
+__device__ __forceinline__ void group_barrier(int hg) {  // the four epilogue warps of a column group
   asm volatile("bar.sync %0, 128;" ::"r"(1 + hg) : "memory");
 }
 
-// HC: 16-column chunks of a column half kept in registers (the sum over the K
+// ---- output head: R token rows over a 128-id vocabulary tile.  Lane l
+// holds ids 4l..4l+3 of each row; `masked` has a bit for each of them that is
+// suppressed or past the vocabulary.  Reductions over the warp run on integer
+// keys in the order of the floats (redux.sync), lowest id on ties; the
+// rows go through each stage together so that its latencies overlap.
+
+// Order-preserving key of a float; 0 (below every number) for NaN, and one
+// key for both zeros.
+__device__ __forceinline__ uint32_t order_key(float x) {
+  const uint32_t u = __float_as_uint(x + 0.f);
+  return x != x ? 0u : u ^ (static_cast<uint32_t>(static_cast<int32_t>(u) >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float key_value(uint32_t k) {
+  return k == 0u ? -INFINITY : __uint_as_float(k & 0x80000000u ? k ^ 0x80000000u : ~k);
+}
+// The warp's best key and the lowest id of the lanes that hold it.
+__device__ __forceinline__ uint32_t warp_argmax(uint32_t key, int id, int *arg) {
+  const uint32_t b = __reduce_max_sync(0xffffffffu, key);
+  *arg = static_cast<int>(__reduce_min_sync(0xffffffffu, key == b && b != 0u ? static_cast<uint32_t>(id) : 0x7fffffffu));
+  return b;
+}
+
+// Greedy: maximum and lowest id attaining it.
+template <int R>
+__device__ __forceinline__ void head_rows_greedy(const float4 (&z4)[R], uint32_t masked, int id0, HeadRec (&r)[R]) {
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const float z[4] = {masked & 1u ? -INFINITY : z4[k].x, masked & 2u ? -INFINITY : z4[k].y,
+                        masked & 4u ? -INFINITY : z4[k].z, masked & 8u ? -INFINITY : z4[k].w};
+    const float m = fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3]));  // (NaN only if all are)
+    const int id = z[0] == m ? 0 : z[1] == m ? 1 : z[2] == m ? 2 : 3;
+    r[k] = HeadRec{};
+    r[k].m = key_value(warp_argmax(order_key(m), id0 + id, &r[k].arg));
+    r[k].gm = -INFINITY;
+    r[k].garg = 0x7fffffff;
+  }
+}
+
+// Sampling: maximum and sum of exponentials of x = z / T (for the log-sum-exp)
+// and the Gumbel-max draw, argmax x - log(-log u).  The four ids of a lane
+// share one Philox block.  The draw's order is that of the exponential race
+// exp(x) / -log(u), which needs three fast special functions per id; only ids
+// within kRaceTol of the warp's best are scored exactly (one lane, nearly
+// always), so the draw is that of the exact scores of every id.  Estimating
+// exp(x - max) and log u so leaves a relative error below 2^-11: near u = 1,
+// where the fast logarithm loses its relative precision (its absolute error on
+// [1/2, 1] is below 2^-21), -log(u) is t + t^2/2 + O(t^3) with t = 1 - u exact
+// below t = 2^-8, and within 2^-13 above; the exponential and the reciprocal
+// are good to 2^-20 where they matter (an id whose x is 20 below the tile's
+// maximum cannot win: u lies in [2^-24, 1 - 2^-24]).
+// ss[k]: (slot and block row, step) of row k.
+constexpr float kRaceTol = 4e-3f;
+constexpr float kLog2e = 1.4426950408889634f;
+template <int R>
+__device__ __forceinline__ void head_rows_sample(const GemmParams &p, const float4 (&z4)[R], uint32_t masked, int id0,
+                                                 const int2 *ss, HeadRec (&r)[R]) {
+  float z[R][4], u[R][4], e[R][4], w[R][4], zmax[R], sum[R];
+  const float c = __fdiv_rn(kLog2e, p.temperature);
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    z[k][0] = masked & 1u ? -INFINITY : z4[k].x;
+    z[k][1] = masked & 2u ? -INFINITY : z4[k].y;
+    z[k][2] = masked & 4u ? -INFINITY : z4[k].z;
+    z[k][3] = masked & 8u ? -INFINITY : z4[k].w;
+    zmax[k] = key_value(
+        __reduce_max_sync(0xffffffffu, order_key(fmaxf(fmaxf(z[k][0], z[k][1]), fmaxf(z[k][2], z[k][3])))));
+  }
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    const Philox4 o = philox4x32_10(static_cast<uint32_t>(id0) >> 2, static_cast<uint32_t>(ss[k].x) >> 24,
+                                    static_cast<uint32_t>(ss[k].y),
+                                    (p.tag << 24) | (static_cast<uint32_t>(ss[k].x) & 0xFFFFFFu),
+                                    static_cast<uint32_t>(p.seed), static_cast<uint32_t>(p.seed >> 32));
+    sum[k] = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      // word_to_open_uniform's (w >> 9 + 1/2) / 2^23, without a conversion: exact
+      u[k][i] = __uint_as_float((o.x[i] >> 9) | 0x3f800000u) - 0.999999940395355224609375f;
+      const float t = 1.f - u[k][i];
+      w[k][i] = t < 0.00390625f ? t * __fmaf_rn(t, 0.5f * kLog2e, kLog2e) : -lg2f_fast(u[k][i]);
+      e[k][i] = (masked >> i) & 1u ? 0.f : exp2f_fast((z[k][i] - zmax[k]) * c);
+      sum[k] += e[k][i];
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int k = 0; k < R; ++k) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], off);
+  float best[R];
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    r[k] = HeadRec{};
+    r[k].arg = 0x7fffffff;
+    r[k].m = __fdiv_rn(zmax[k], p.temperature);  // = max x: division by T > 0 is monotonic
+    r[k].s = zmax[k] == -INFINITY ? 0.f : sum[k];
+    // the lane's best e / w by cross products (0 in place of NaN), then the
+    // warp's: nonnegative floats are ordered like their bits
+    float be = 0.f, bw = 1.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (e[k][i] * bw > be * w[k][i]) {
+        be = e[k][i];
+        bw = w[k][i];
+      }
+    best[k] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(__fdividef(be, bw))));
+  }
+  // Exact scores of the candidates: each lane's first one of every row
+  // together, further ones (rare) after.
+  uint32_t cand[R], gkey[R];
+  int gid[R];
+  auto take = [&](int k) {  // score row k's lowest candidate of this lane
+    const int i = __ffs(static_cast<int>(cand[k])) - 1;
+    const float zi = i == 0 ? z[k][0] : i == 1 ? z[k][1] : i == 2 ? z[k][2] : z[k][3];
+    const float ui = i == 0 ? u[k][0] : i == 1 ? u[k][1] : i == 2 ? u[k][2] : u[k][3];
+    const float x = __fdiv_rn(zi, p.temperature) - logf(-logf(ui));
+    const uint32_t key = i < 0 ? 0u : order_key((masked >> i) & 1u ? -INFINITY : x);
+    if (key > gkey[k]) {
+      gkey[k] = key;
+      gid[k] = id0 + i;
+    }
+    cand[k] &= cand[k] - 1;
+  };
+  uint32_t more = 0;
+#pragma unroll
+  for (int k = 0; k < R; ++k) {
+    // without a finite maximum every id is scored; a masked id scores -inf, so
+    // that a row without any other id has one
+    const bool all = !(fabsf(zmax[k]) <= 3.402823466e38f);
+    const float floor = best[k] - best[k] * kRaceTol;
+    cand[k] = masked;
+    gid[k] = 0x7fffffff;
+    gkey[k] = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (all || e[k][i] >= floor * w[k][i]) cand[k] |= 1u << i;
+    take(k);
+    more |= cand[k];
+  }
+  while (__any_sync(0xffffffffu, more)) {
+    more = 0;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      take(k);
+      more |= cand[k];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < R; ++k) r[k].gm = key_value(warp_argmax(gkey[k], gid[k], &r[k].garg));
+}
+
+// HC: 16-column chunks of a column group kept in registers (the sum over the K
 // chunks); 0: no split (p.splits == 1), the epilogue reads TMEM directly.
 template <int EPI, int HC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads<EPI>, 1)
     gemm_wide_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                      const GemmParams p) {
+  constexpr int kEW = kWideEpiWarps<EPI>, kGroups = kEW / 4;
+  constexpr int kSlice = 32 / kGroups;  // token rows per staging buffer
+  constexpr int kR = kSlice / 4;        // of them a warp's
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t *smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);
@@ -78,7 +242,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
   // (even CTA: the stage's tiles of both CTAs landed)
   uint64_t *empty = full + kWideMaxStages;   // the MMAs that read the stage completed
   uint64_t *accf = empty + kWideMaxStages;   // accumulator holds a finished chunk
-  uint64_t *acce = accf + 2;                 // even CTA: all 16 epilogue warps are done with it
+  uint64_t *acce = accf + 2;                 // even CTA: all epilogue warps of the pair are done with it
   uint64_t *done = acce + 2;                 // even CTA: every MMA completed
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
   volatile int &s_timed_out = *reinterpret_cast<int *>(tmem_slot + 1);
@@ -101,7 +265,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&accf[a], 1);
-      mbar_init(&acce[a], 16);
+      mbar_init(&acce[a], 2 * kEW);
     }
     mbar_init(done, 1);
     fence_barrier_init();
@@ -217,48 +381,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
     if (!ok) s_timed_out = 1;
     if (elect_one()) umma_commit_pair(done, 1);
   } else if (warp >= kWideEpiWarp) {
-    // ---------------- epilogue: warp -> lane quarter (its TMEM rows), column half
+    // ---------------- epilogue: warp -> lane quarter (its TMEM rows), column group
     const int ew = warp - kWideEpiWarp, quarter = warp & 3, hg = ew >> 2;
-    const int half = BT / 2;  // columns of this warp's half
-    const int n_sl = half / kWideSlice;
-    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + hg * half;
+    const int gcols = BT / kGroups;  // columns of this warp's group
+    const int n_sl = gcols / kSlice;
+    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + hg * gcols;
     const uint32_t acce_u32[2] = {dsmem_map(smem_u32(&acce[0]), 0), dsmem_map(smem_u32(&acce[1]), 0)};
     const int feat = quarter * 32 + lane;  // this thread's feature of the 128
-    float *buf0 = stg + hg * 2 * kWideSlice * 128;
+    float *buf0 = stg + hg * 2 * kSlice * 128;
     const int stat_tiles = p.N / 128;
     bool ok = true;
     int q = 0;
     pdl_wait();
-    int par = 0;
+    int par = 0, n_written = 0;
     for (int tile = pair; tile < tiles; tile += n_pairs, par ^= 1) {
       const int ntile = (tile / p.n_tt) * 2 + rank, n0 = ntile * 128;
-      const int th = (tile % p.n_tt) * BT + hg * half;  // first token row of the half
-      int2 *tk = tok + par * 256 + hg * 128;
-      if constexpr (EPI == EPI_KV) {
-        // (slot, position) of the half's rows; the first slice's barrier
-        // publishes them
+      const int th = (tile % p.n_tt) * BT + hg * gcols;  // first token row of the group
+      int2 *tk = tok + par * 256 + hg * (256 / kGroups);
+      if constexpr (EPI == EPI_KV || EPI == EPI_HEAD) {
+        // (slot, position) of the group's rows, or for a sampling head (slot
+        // and row of the block in the top byte, step); the first slice's
+        // barrier publishes them
         const int j = (ew & 3) * 32 + lane, t = th + j;
         int2 sp = make_int2(0, 0x7fffffff);
-        if (j < half && t < p.M) {
+        if (j < gcols && t < p.M && (EPI == EPI_KV || p.temperature > 0.f)) {
           const int i = t / p.rows_per_seq, jr = t - i * p.rows_per_seq;
           sp.x = p.seq_slot[i];
-          sp.y = (p.pos_base ? p.pos_base[sp.x] : 0) + jr;
+          if constexpr (EPI == EPI_KV) {
+            sp.y = (p.pos_base ? p.pos_base[sp.x] : 0) + jr;
+          } else {
+            sp.y = p.step[sp.x];
+            sp.x |= jr << 24;
+          }
         }
-        tk[j] = sp;
+        if (j < gcols) tk[j] = sp;
       }
-      float b4[4];
+      float b4[4] = {0.f, 0.f, 0.f, 0.f};
+      uint32_t masked = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int nn = n0 + 4 * lane + i;
-        b4[i] = (p.bias && nn < p.N) ? bf2f(p.bias[nn]) : 0.f;
+        if constexpr (EPI == EPI_HEAD) masked |= (nn >= p.N || (p.suppress && p.suppress[nn])) ? 1u << i : 0u;
+        else b4[i] = (p.bias && nn < p.N) ? bf2f(p.bias[nn]) : 0.f;
       }
       // the residual rows of a slice (this warp's four), loaded ahead of use
-      float4 old[4];
+      float4 old[kR];
       auto load_old = [&](int sl) {
         if constexpr (EPI == EPI_RESID) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int t = th + sl * kWideSlice + quarter * 4 + k;
+          for (int k = 0; k < kR; ++k) {
+            const int t = th + sl * kSlice + quarter * kR + k;
             old[k] = (t < p.M && n0 < p.N)
                          ? *reinterpret_cast<const float4 *>(p.resid + static_cast<size_t>(t) * p.ld_resid + n0 + 4 * lane)
                          : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -301,23 +473,50 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
       }
       if (!ok) s_timed_out = 1;
 
-      // slices of 16 token rows through shared memory: a warp then owns whole
+      // slices of token rows through shared memory: a warp then owns whole
       // rows (lane l: features 4l..4l+3), so stores are full lines and the
       // row's LayerNorm statistics over the 128 features are warp reductions
-      auto slice = [&](int sl, const float *src16) {
-        float *buf = buf0 + (sl & 1) * kWideSlice * 128;
+      auto slice = [&](int sl, const float *src) {
+        // the two buffers alternate over all slices, whatever a tile's number
+        // of them: a slice's barrier says that the one before has been read
+        float *buf = buf0 + (n_written++ & 1) * kSlice * 128;
 #pragma unroll
-        for (int jj = 0; jj < 16; ++jj) buf[jj * 128 + feat] = src16[jj];
-        half_barrier(hg);
-        float4 cur[4];
+        for (int jj = 0; jj < kSlice; ++jj) buf[jj * 128 + feat] = src[jj];
+        group_barrier(hg);
+        if constexpr (EPI == EPI_HEAD) {
+          const int j0 = quarter * kR, tl0 = sl * kSlice + j0;
+          if (!ok || th + tl0 >= p.M || n0 >= p.N) return;
+          float4 z4[kR];
+          HeadRec r[kR];
+#pragma unroll
+          for (int k = 0; k < kR; ++k) z4[k] = *reinterpret_cast<const float4 *>(buf + (j0 + k) * 128 + 4 * lane);
+          if (p.logits) {
+#pragma unroll
+            for (int k = 0; k < kR; ++k) {
+              if (th + tl0 + k >= p.M) break;
+              float *lrow = p.logits + static_cast<size_t>(th + tl0 + k) * p.N + n0;
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                if (n0 + i * 32 + lane < p.N) lrow[i * 32 + lane] = buf[(j0 + k) * 128 + i * 32 + lane];
+            }
+          }
+          if (p.temperature > 0.f) head_rows_sample(p, z4, masked, n0 + 4 * lane, tk + tl0, r);
+          else head_rows_greedy(z4, masked, n0 + 4 * lane, r);
+#pragma unroll
+          for (int k = 0; k < kR; ++k)
+            if (lane == k && th + tl0 + k < p.M)
+              p.recs[static_cast<size_t>(th + tl0 + k) * ((p.N + 127) / 128) + ntile] = r[k];
+          return;
+        }
+        float4 cur[kR];
         if constexpr (EPI == EPI_RESID) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k) cur[k] = old[k];
+          for (int k = 0; k < kR; ++k) cur[k] = old[k];
           if (sl + 1 < n_sl) load_old(sl + 1);
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int jr = quarter * 4 + k, tl = sl * kWideSlice + jr, t = th + tl;
+        for (int k = 0; k < kR; ++k) {
+          const int jr = quarter * kR + k, tl = sl * kSlice + jr, t = th + tl;
           const bool valid = ok && t < p.M && n0 < p.N;
           const float4 a4 = *reinterpret_cast<const float4 *>(buf + jr * 128 + 4 * lane);
           const float v[4] = {a4.x + b4[0], a4.y + b4[1], a4.z + b4[2], a4.w + b4[3]};
@@ -354,9 +553,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads, 1)
       } else {
         const uint32_t src = trow + (q & 1) * kWideAcc;
         for (int c = 0; c < n_sl; ++c) {
-          float v[16];
-          tmem_ld16_issue(src + c * 16, v);
-          tmem_ld_wait(v);
+          float v[kSlice];
+          tmem_ld<kSlice>(src + c * kSlice, v);
           if (c + 1 == n_sl) {
             tc_fence_before();
             __syncwarp();
@@ -420,6 +618,7 @@ static cudaError_t gemm_wide_init() {
     if (status == cudaSuccess) status = wide_attr<EPI_KV, 4>();
     if (status == cudaSuccess) status = wide_attr<EPI_KV, 0>();
     if (status == cudaSuccess) status = wide_attr<EPI_F32, 0>();
+    if (status == cudaSuccess) status = wide_attr<EPI_HEAD, 0>();
   });
   return status;
 }
@@ -428,7 +627,7 @@ static cudaError_t gemm_wide_init() {
 // take the shape.
 static bool gemm_wide_plan(GemmParams &p, size_t *smem, int *pairs) {
   if (p.M <= 0 || p.N <= 0 || p.K <= 0 || p.K % 64 || p.ln_x) return false;
-  if (p.splits < 1) p.splits = 1;
+  if (p.splits < 1 || p.epi == EPI_HEAD) p.splits = 1;
   const int k_iters = p.K / 64;
   if (k_iters % p.splits) return false;
   p.kps = k_iters / p.splits;
@@ -440,7 +639,7 @@ static bool gemm_wide_plan(GemmParams &p, size_t *smem, int *pairs) {
     return n;
   }();
   if (n_sm < 2) return false;
-  const bool direct = p.splits == 1 && (p.epi == EPI_KV || p.epi == EPI_F32);
+  const bool direct = p.splits == 1 && (p.epi == EPI_KV || p.epi == EPI_F32 || p.epi == EPI_HEAD);
   const int max_bt = direct ? 256 : 128, n_nt = (p.N + 255) / 256, slots = n_sm / 2;
   // The token tile with the least estimated time: per tile the larger of its
   // MMAs and its operand fetch (64 bytes per cycle and SM) over the k-steps
@@ -453,7 +652,10 @@ static bool gemm_wide_plan(GemmParams &p, size_t *smem, int *pairs) {
     const long long tiles = static_cast<long long>(n_tt) * n_nt;
     const long long waves = (tiles + slots - 1) / slots;
     const long long fetch = (128 + bt / 2) * 2, mma = 2 * bt;
-    const long long cost = waves * (k_iters * (fetch > mma ? fetch : mma) + 12 * bt);
+    const long long steps = k_iters * (fetch > mma ? fetch : mma);
+    // (a head's epilogue of a tile runs under the next tile's MMAs)
+    const long long head = (p.temperature > 0.f ? 70 : 20) * bt;
+    const long long cost = p.epi == EPI_HEAD ? waves * (steps > head ? steps : head) + head : waves * (steps + 12 * bt);
     if (p.BT == 0 || cost < best) {
       best = cost;
       p.BT = bt;
@@ -476,7 +678,7 @@ static cudaError_t wide_launch(const CUtensorMap *tw, const CUtensorMap *tx, con
                                int pairs, cudaStream_t s, bool pdl) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(kWideThreads);
+  cfg.blockDim = dim3(kWideThreads<EPI>);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -507,6 +709,7 @@ cudaError_t launch_gemm_wide(const void *X, const void *W, GemmParams p, cudaStr
     case EPI_KV:
       return direct ? wide_launch<EPI_KV, 0>(tw, tx, p, smem, pairs, s, pdl)
                     : wide_launch<EPI_KV, 4>(tw, tx, p, smem, pairs, s, pdl);
+    case EPI_HEAD: return wide_launch<EPI_HEAD, 0>(tw, tx, p, smem, pairs, s, pdl);
   }
   return cudaErrorInvalidValue;
 }

@@ -75,3 +75,43 @@ def test_step_rows_do_not_depend_on_batch(n):
             for i in (pair[0], pair[0] + 3 * ((n - 3) // 3)):
                 assert torch.equal(a[i], b[0])
                 assert torch.equal(a[i + pair[1] - pair[0]], b[1])
+
+
+@pytest.mark.parametrize("T,mask", [(0.25, False), (0.7, True), (1.0, False), (30.0, True)])
+def test_sampling_head_draws_the_exact_argmax(T, mask):
+    """The head's Gumbel-max draw (ids screened by an estimate, the survivors
+    scored exactly) is the argmax of x + G over every id that is not
+    suppressed, on the GPU's own logits with the oracle's noise, wherever the
+    two best scores differ by more than the logarithms' rounding (1e-4 at
+    scores below 20).  Odd vocabulary, whole vocabulary tiles suppressed."""
+    import torch
+    from oracle import philox
+    from paper_2609_32869_gb300 import binding as B
+    from paper_2609_32869_gb300.session import Session, upload_weights
+    cfg, n, seed = syn.TINY, 13, 77
+    K, V = cfg.block_k, cfg.vocab
+    dev = upload_weights(syn.make_weights(cfg, seed=4))
+    enc = syn.encoder_output(cfg, 1, seed=2)[np.zeros(n, int)]
+    prompt = syn.prompts(cfg, n, length=5, seed=3)
+    sup = np.zeros(V, np.uint8)
+    if mask:
+        sup[syn.uniform_int(5, "sup", (V // 3,), 0, V - 1)] = 1
+        sup[128:384] = 1
+    d_sup = torch.from_numpy(sup).cuda()
+    sp = B.sample_params(T, seed, d_sup if mask else None)
+    s = Session(cfg, dev, max_batch=n, keep_logits=True)
+    s.prefill(np.arange(n, dtype=np.int32), enc, prompt, np.full(n, 60, np.int32))
+    s.draft(sp=sp)
+    z = s.view(B.WF_VIEW_DRAFT_LOGITS, torch.float32, (n, K + 1, V)).cpu().numpy()
+    cand = s.view(B.WF_VIEW_CANDIDATES, torch.int32, (n, K)).cpu().numpy()
+    clear = 0
+    for i in range(n):
+        for j in range(1, K + 1):
+            x = z[i, j] / np.float32(T) + philox.gumbel_noise(seed, i, 1, j, philox.TAG_DRAFT, V)
+            x[sup != 0] = -np.inf
+            top = np.argsort(x)[-2:]
+            if x[top[1]] - x[top[0]] > 1e-4:
+                assert cand[i, j - 1] == top[1], (i, j)
+                clear += 1
+    assert clear > n * K // 2 and s.error() == 0
+    s.close()
