@@ -42,7 +42,6 @@ constexpr int kDPT = kQG * 64 / kThreadsA;  // output dims per thread in the com
 constexpr int kPartStride = 2 + 64;   // m, l, o[64]
 // Scores are kept in base-2 units (times log2 e): every softmax weight, and
 // every weight of the merges of partial results, is one exp2.
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kSmemK = kKB * 128;     // bytes
 constexpr int kSmemQ = kQG * 128;
 // K, V, Q, then the warps' (m, l); the warps' O partials reuse the K tile.

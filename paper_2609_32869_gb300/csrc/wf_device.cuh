@@ -97,13 +97,31 @@ __device__ __forceinline__ void mbar_drain(uint64_t *bar, uint32_t parity) {
   while (!mbar_try_wait(bar, parity) && clock64() - t0 < kSpinLimitCycles) {
   }
 }
+// One look at a phase, without waiting.
+__device__ __forceinline__ uint32_t mbar_test(uint64_t *bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok;
+}
+// A try_wait may suspend the thread for longer than a very short limit; below
+// this many cycles the waits look without suspending, so that the limit holds.
+constexpr long long kSuspendCycles = 10000;
+__device__ __forceinline__ uint32_t mbar_poll(uint64_t *bar, uint32_t parity, long long limit) {
+  return limit < kSuspendCycles ? mbar_test(bar, parity) : mbar_try_wait(bar, parity);
+}
 // Bounded wait on a phase of an mbarrier.  Returns false (and sets the error
 // word) if the phase did not complete within `limit` clock cycles.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t *err,
                                           long long limit) {
-  if (mbar_try_wait(bar, parity)) return true;
-  long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
+  if (mbar_test(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_poll(bar, parity, limit)) {
     if (clock64() - t0 > limit) {
       set_error(err, WF_DEV_ERR_TIMEOUT);
       return false;
@@ -114,8 +132,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32
 
 // mbar_wait by a converged warp: every lane waits, one answer.
 __device__ __forceinline__ bool warp_mbar_wait(uint64_t *bar, uint32_t parity, uint32_t *err, long long limit) {
+  if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
   const long long t0 = clock64();
-  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+  while (!__all_sync(0xffffffffu, mbar_poll(bar, parity, limit))) {
     if (__any_sync(0xffffffffu, clock64() - t0 > limit)) {
       set_error(err, WF_DEV_ERR_TIMEOUT);
       return false;
@@ -499,6 +518,31 @@ __device__ __forceinline__ float gumbel(uint64_t seed, uint32_t seq, uint32_t st
                             static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32));
   const float u = word_to_open_uniform(o.x[v & 3]);
   return -logf(-logf(u));
+}
+
+// Order-preserving key of a float; 0 (below every number) for NaN, and one
+// key for both zeros.
+__device__ __forceinline__ uint32_t order_key(float x) {
+  const uint32_t u = __float_as_uint(x + 0.f);
+  return x != x ? 0u : u ^ (static_cast<uint32_t>(static_cast<int32_t>(u) >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float key_value(uint32_t k) {
+  return k == 0u ? -INFINITY : __uint_as_float(k & 0x80000000u ? k ^ 0x80000000u : ~k);
+}
+
+// Gumbel-max draws are screened by the exponential race: argmax x - log(-log u)
+// is argmax exp(x) / -log u, whose estimate takes a few fast instructions.
+// neg_log2_estimate is -log2 u within a relative 2^-12: near u = 1, where the
+// fast logarithm (absolute error below 2^-21 on [1/2, 1]) loses its relative
+// precision, -log u is t + t^2/2 + O(t^3) with t = 1 - u exact.  With the
+// division (and, in the head, an exponential) an estimated score is within
+// 2^-10 of the true one, so an id that scores best exactly is never more than
+// kRaceTol below the best estimate.
+constexpr float kRaceTol = 4e-3f;
+constexpr float kLog2e = 1.4426950408889634f;
+__device__ __forceinline__ float neg_log2_estimate(float u) {
+  const float t = 1.f - u;
+  return t < 0.00390625f ? t * __fmaf_rn(t, 0.5f * kLog2e, kLog2e) : -lg2f_fast(u);
 }
 
 }  // namespace wf

@@ -77,15 +77,6 @@ __device__ __forceinline__ void group_barrier(int hg) {  // the four epilogue wa
 // keys in the order of the floats (redux.sync), lowest id on ties; the
 // rows go through each stage together so that its latencies overlap.
 
-// Order-preserving key of a float; 0 (below every number) for NaN, and one
-// key for both zeros.
-__device__ __forceinline__ uint32_t order_key(float x) {
-  const uint32_t u = __float_as_uint(x + 0.f);
-  return x != x ? 0u : u ^ (static_cast<uint32_t>(static_cast<int32_t>(u) >> 31) | 0x80000000u);
-}
-__device__ __forceinline__ float key_value(uint32_t k) {
-  return k == 0u ? -INFINITY : __uint_as_float(k & 0x80000000u ? k ^ 0x80000000u : ~k);
-}
 // The warp's best key and the lowest id of the lanes that hold it.
 __device__ __forceinline__ uint32_t warp_argmax(uint32_t key, int id, int *arg) {
   const uint32_t b = __reduce_max_sync(0xffffffffu, key);
@@ -114,16 +105,10 @@ __device__ __forceinline__ void head_rows_greedy(const float4 (&z4)[R], uint32_t
 // share one Philox block.  The draw's order is that of the exponential race
 // exp(x) / -log(u), which needs three fast special functions per id; only ids
 // within kRaceTol of the warp's best are scored exactly (one lane, nearly
-// always), so the draw is that of the exact scores of every id.  Estimating
-// exp(x - max) and log u so leaves a relative error below 2^-11: near u = 1,
-// where the fast logarithm loses its relative precision (its absolute error on
-// [1/2, 1] is below 2^-21), -log(u) is t + t^2/2 + O(t^3) with t = 1 - u exact
-// below t = 2^-8, and within 2^-13 above; the exponential and the reciprocal
-// are good to 2^-20 where they matter (an id whose x is 20 below the tile's
-// maximum cannot win: u lies in [2^-24, 1 - 2^-24]).
+// always), so the draw is that of the exact scores of every id.  (An id whose x is 20 below
+// the tile's maximum cannot win, as u lies in [2^-24, 1 - 2^-24], so the fast
+// exponential is good to 2^-20 wherever it matters.)
 // ss[k]: (slot and block row, step) of row k.
-constexpr float kRaceTol = 4e-3f;
-constexpr float kLog2e = 1.4426950408889634f;
 template <int R>
 __device__ __forceinline__ void head_rows_sample(const GemmParams &p, const float4 (&z4)[R], uint32_t masked, int id0,
                                                  const int2 *ss, HeadRec (&r)[R]) {
@@ -149,8 +134,7 @@ __device__ __forceinline__ void head_rows_sample(const GemmParams &p, const floa
     for (int i = 0; i < 4; ++i) {
       // word_to_open_uniform's (w >> 9 + 1/2) / 2^23, without a conversion: exact
       u[k][i] = __uint_as_float((o.x[i] >> 9) | 0x3f800000u) - 0.999999940395355224609375f;
-      const float t = 1.f - u[k][i];
-      w[k][i] = t < 0.00390625f ? t * __fmaf_rn(t, 0.5f * kLog2e, kLog2e) : -lg2f_fast(u[k][i]);
+      w[k][i] = neg_log2_estimate(u[k][i]);
       e[k][i] = (masked >> i) & 1u ? 0.f : exp2f_fast((z[k][i] - zmax[k]) * c);
       sum[k] += e[k][i];
     }

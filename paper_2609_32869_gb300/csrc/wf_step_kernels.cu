@@ -52,25 +52,34 @@ __global__ void embed_kernel(const EmbedParams p) {
   float *x = p.x + static_cast<size_t>(r) * p.d;
   // thread tid holds feature 128k + tid of every 128-feature tile k
   const int tiles = p.d >> 7;
+  // every load before the first store: the row's latencies overlap (11 us a
+  // launch when each tile's stores stood between its loads and the next's)
   float v[kMaxStatTiles];
+  bf16 emb[kMaxStatTiles], pe[kMaxStatTiles], gn[kMaxStatTiles], bn[kMaxStatTiles];
+  const bf16 *src = use_mask ? p.mask_emb : p.tok_emb + static_cast<size_t>(tok) * p.d;
+  const bf16 *psrc = use_mask || p.drafter ? nullptr : p.pos_emb + static_cast<size_t>(pos) * p.d;
 #pragma unroll
   for (int k = 0; k < kMaxStatTiles; ++k) {
     if (k >= tiles) continue;
     const int e = k * 128 + threadIdx.x;
-    float val;
-    if (use_mask) {
-      val = bf2f(p.mask_emb[e]);
-    } else {
-      val = bf2f(p.tok_emb[static_cast<size_t>(tok) * p.d + e]);
-      if (!p.drafter) val += bf2f(p.pos_emb[static_cast<size_t>(pos) * p.d + e]);
-    }
+    emb[k] = src[e];
+    if (psrc) pe[k] = psrc[e];
+    if (p.xg) gn[k] = p.g_next[e];
+    if (p.xg && r == 0) bn[k] = p.b_next[e];
+  }
+#pragma unroll
+  for (int k = 0; k < kMaxStatTiles; ++k) {
+    if (k >= tiles) continue;
+    const int e = k * 128 + threadIdx.x;
+    float val = bf2f(emb[k]);
+    if (psrc) val += bf2f(pe[k]);
     v[k] = val;
     x[e] = val;
     if (p.xg) {
-      p.xg[static_cast<size_t>(r + 2) * p.d + e] = __float2bfloat16(val * bf2f(p.g_next[e]));
+      p.xg[static_cast<size_t>(r + 2) * p.d + e] = __float2bfloat16(val * bf2f(gn[k]));
       if (r == 0) {
-        p.xg[e] = p.g_next[e];
-        p.xg[static_cast<size_t>(p.d) + e] = p.b_next[e];
+        p.xg[e] = gn[k];
+        p.xg[static_cast<size_t>(p.d) + e] = bn[k];
       }
     }
   }
@@ -221,53 +230,91 @@ cudaError_t launch_layernorm(const float *x, const float2 *stats, int in_stride,
 }
 
 // ---------------------------------------------------------- head reduce --
-// Combine the per-tile records of each row in tile order (deterministic):
-// argmax with the lowest id on ties, log-sum-exp, and the Gumbel-max draw.
-__device__ __forceinline__ void rec_combine(float &m, float &s, int &arg, float &gm, int &garg,
-                                            const HeadRec &r) {
-  const float M = fmaxf(m, r.m);
-  float ns = 0.f;
-  if (M != -INFINITY)
-    ns = (m == -INFINITY ? 0.f : s * __expf(m - M)) + (r.m == -INFINITY ? 0.f : r.s * __expf(r.m - M));
-  if (r.m > m || (r.m == m && r.arg < arg)) arg = r.arg;
-  m = M;
-  s = ns;
-  if (r.gm > gm || (r.gm == gm && r.garg < garg)) {
-    gm = r.gm;
-    garg = r.garg;
-  }
-}
-
-__global__ void head_reduce_kernel(const HeadReduceParams p) {
+// Combine the per-tile records of each row: argmax (or Gumbel-max draw) with
+// the lowest id on ties, and when sampling the log-sum-exp.  One CTA per row,
+// every record of a thread in flight at once (a warp per row that folded its
+// records one by one took 14 us, all of it load latency).  The order of the
+// sum depends on the vocabulary only.
+constexpr int kRedThreads = 128;
+constexpr int kRedUnroll = 4;  // records per thread and round: 512 tiles, 65536 ids
+__global__ void __launch_bounds__(kRedThreads) head_reduce_kernel(const HeadReduceParams p) {
   pdl_wait();
   pdl_launch_dependents();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (warp >= p.rows) return;
-  const HeadRec *rr = p.recs + static_cast<size_t>(warp) * p.n_tiles;
-  // lane l reduces tiles l, l+32, ... in order; lanes then combine in order
-  float m = -INFINITY, s = 0.f, gm = -INFINITY;
-  int arg = 0x7fffffff, garg = 0x7fffffff;
-  for (int t = lane; t < p.n_tiles; t += 32) rec_combine(m, s, arg, gm, garg, rr[t]);
-  for (int off = 1; off < 32; off <<= 1) {
-    HeadRec o;
-    o.m = __shfl_down_sync(0xffffffffu, m, off);
-    o.s = __shfl_down_sync(0xffffffffu, s, off);
-    o.gm = __shfl_down_sync(0xffffffffu, gm, off);
-    o.arg = __shfl_down_sync(0xffffffffu, arg, off);
-    o.garg = __shfl_down_sync(0xffffffffu, garg, off);
-    if ((lane & (2 * off - 1)) == 0 && lane + off < 32) rec_combine(m, s, arg, gm, garg, o);
+  __shared__ float s_best[kRedThreads / 32], s_m[kRedThreads / 32], s_s[kRedThreads / 32];
+  __shared__ int s_id[kRedThreads / 32];
+  const int row = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const HeadRec *rr = p.recs + static_cast<size_t>(row) * p.n_tiles;
+  float best = -INFINITY, m = -INFINITY, sum = 0.f;
+  int id = 0x7fffffff;
+  for (int t0 = tid; t0 < p.n_tiles; t0 += kRedThreads * kRedUnroll) {
+    float rm[kRedUnroll], rs[kRedUnroll], rg[kRedUnroll];
+    int ri[kRedUnroll];
+#pragma unroll
+    for (int i = 0; i < kRedUnroll; ++i) {
+      const int t = t0 + i * kRedThreads;
+      rm[i] = rg[i] = -INFINITY;
+      rs[i] = 0.f;
+      ri[i] = 0x7fffffff;
+      if (t < p.n_tiles) {
+        rm[i] = rr[t].m;
+        rs[i] = rr[t].s;
+        rg[i] = p.sampling ? rr[t].gm : rm[i];
+        ri[i] = p.sampling ? rr[t].garg : rr[t].arg;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kRedUnroll; ++i) {
+      if (rg[i] > best || (rg[i] == best && ri[i] < id)) {
+        best = rg[i];
+        id = ri[i];
+      }
+      if (p.sampling) {
+        const float M = fmaxf(m, rm[i]);
+        if (M != -INFINITY)
+          sum = (m == -INFINITY ? 0.f : sum * __expf(m - M)) + (rm[i] == -INFINITY ? 0.f : rs[i] * __expf(rm[i] - M));
+        m = M;
+      }
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const float b2 = __shfl_xor_sync(0xffffffffu, best, off);
+    const int i2 = __shfl_xor_sync(0xffffffffu, id, off);
+    if (b2 > best || (b2 == best && i2 < id)) {
+      best = b2;
+      id = i2;
+    }
+  }
+  if (p.sampling) {
+    const float M = key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
+    sum = warp_sum(m == -INFINITY ? 0.f : sum * __expf(m - M));
+    m = M;
   }
   if (lane == 0) {
+    s_best[warp] = best;
+    s_id[warp] = id;
+    s_m[warp] = m;
+    s_s[warp] = sum;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    float M = -INFINITY, S = 0.f;
+    for (int w = 0; w < kRedThreads / 32; ++w) {
+      if (w > 0 && (s_best[w] > best || (s_best[w] == best && s_id[w] < id))) {
+        best = s_best[w];
+        id = s_id[w];
+      }
+      M = fmaxf(M, s_m[w]);
+    }
+    for (int w = 0; w < kRedThreads / 32; ++w) S += s_m[w] == -INFINITY ? 0.f : s_s[w] * __expf(s_m[w] - M);
     HeadOut out;
-    out.arg = arg;
-    out.garg = garg;
-    out.m = m;
-    out.lse = m + logf(s);
-    p.out[warp] = out;
+    out.arg = out.garg = id;  // the one its reader asks for (greedy or sampling)
+    out.m = p.sampling ? M : best;
+    out.lse = p.sampling ? M + logf(S) : 0.f;
+    p.out[row] = out;
     if (p.cand) {
-      const int i = warp / p.rps, j = warp - i * p.rps;
-      if (j >= 1 && j <= p.K) p.cand[p.seq_slot[i] * p.K + j - 1] = p.sampling ? garg : arg;
+      const int i = row / p.rps, j = row - i * p.rps;
+      if (j >= 1 && j <= p.K) p.cand[p.seq_slot[i] * p.K + j - 1] = id;
     }
   }
 }
@@ -275,23 +322,28 @@ __global__ void head_reduce_kernel(const HeadReduceParams p) {
 cudaError_t launch_head_reduce(const HeadReduceParams &p0, cudaStream_t s, bool pdl) {
   HeadReduceParams p = p0;
   void *args[] = {&p};
-  const int threads = 256;
-  return launch_ex(reinterpret_cast<const void *>(head_reduce_kernel),
-                   dim3((p.rows * 32 + threads - 1) / threads), dim3(threads), args, s, pdl);
+  return launch_ex(reinterpret_cast<const void *>(head_reduce_kernel), dim3(p.rows), dim3(kRedThreads), args, s, pdl);
 }
 
 // --------------------------------------------------------------- accept --
-// One CTA per active sequence.  Greedy (Sec. 3.1): keep proposals while they
+// One CTA per active sequence (greedy) or a cluster of kAccCluster (sampling).  Greedy (Sec. 3.1): keep proposals while they
 // equal the target's argmax, then emit the target's token (correction, or
 // bonus after K agreements).  Sampling (Sec. 3.1, App. A.4): accept c_i when
 // u_i < p_i(c_i)/q_i(c_i) in FP32; at the first rejection draw from the
 // normalised residual (p_i - q_i)_+ by Gumbel-max; after a full block emit
 // the bonus drawn from the target.  An accepted EOS ends the transcript
 // without a bonus; with R tokens left at most R-1 proposals are live; the
-// cache keeps L+1+a positions (App. A.1).  The decisions are sequential and
-// taken by one thread; the residual draw and the normalisers of forced
-// proposal distributions reduce over the vocabulary with the whole CTA.
+// cache keeps L+1+a positions (App. A.1).  One thread per proposal forms its
+// decision and one reads them in order; the residual draw splits the
+// vocabulary over the cluster, and each CTA takes one of the normalisers of
+// forced proposal distributions.  The draw is bound by its arithmetic: one CTA
+// that scored every id (three logarithms and a Philox block each) took 250 us
+// at 51866 ids.  Here a Philox block serves its four ids, and a warp ranks them
+// by the exponential race r / -log u (r the residual, exactly as scored) and
+// scores only ids within kRaceTol of its best so far, so the draw is the exact
+// scores' argmax: 26 us at 32 sequences.
 constexpr int kAccThreads = 256;
+constexpr int kAccCluster = 8;
 
 // The CTA's maximum (value, lowest id on ties) of (v, arg) over its threads.
 __device__ __forceinline__ void block_argmax(float &v, int &arg, float *sv, int *sa) {
@@ -345,43 +397,50 @@ __device__ __forceinline__ float block_lse(float m, float sum, float *sm, float 
   return M + logf(S);
 }
 
+template <int C>  // CTAs per sequence
 __global__ void __launch_bounds__(kAccThreads) accept_kernel(const AcceptParams p) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ float s_v[kAccThreads / 32], s_w[kAccThreads / 32];
   __shared__ int s_a[kAccThreads / 32];
   __shared__ float s_qlse[8];
-  __shared__ int s_em[16];
+  __shared__ int s_em[16], s_cand[8], s_acc[8];
   __shared__ int s_state[4];  // emitted count, accepted a, stopped, rejected row (0: none)
+  __shared__ float s_cv[C];   // the cluster's best scores and their ids (-1: nothing to draw from)
+  __shared__ int s_ca[C];
   const int Kp1 = p.K + 1;
   const int tid = threadIdx.x;
+  const int rank = C > 1 ? static_cast<int>(blockIdx.x % C) : 0, i = blockIdx.x / C, n_ctas = gridDim.x / C;
   // slots outside the active list emit nothing this step
-  for (int sl = blockIdx.x; sl < p.max_batch; sl += gridDim.x) {
-    bool active = false;
-    for (int i = 0; i < p.n_seq; ++i) active = active || p.seq_slot[i] == sl;
-    if (!active) {
-      for (int j = tid; j < Kp1; j += kAccThreads) p.out_tokens[sl * Kp1 + j] = -1;
-      if (tid == 0) p.out_count[sl] = 0;
+  if (rank == 0) {
+    for (int sl = i; sl < p.max_batch; sl += n_ctas) {
+      bool mine = false;
+      for (int q = tid; q < p.n_seq; q += kAccThreads) mine = mine || p.seq_slot[q] == sl;
+      if (!__syncthreads_or(mine)) {
+        for (int j = tid; j < Kp1; j += kAccThreads) p.out_tokens[sl * Kp1 + j] = -1;
+        if (tid == 0) p.out_count[sl] = 0;
+      }
     }
   }
-  const int i = blockIdx.x;
   if (i >= p.n_seq) return;
   const int slot = p.seq_slot[i];
-  if (p.done[slot]) {
-    for (int j = tid; j < Kp1; j += kAccThreads) p.out_tokens[slot * Kp1 + j] = -1;
-    if (tid == 0) p.out_count[slot] = 0;
+  const int finished_before = p.done[slot], R = p.remaining[slot], step = p.step[slot], L0 = p.L[slot];
+  if (C > 1) cluster_sync();  // every CTA has read the state that CTA 0 rewrites
+  if (finished_before) {
+    if (rank == 0) {
+      for (int j = tid; j < Kp1; j += kAccThreads) p.out_tokens[slot * Kp1 + j] = -1;
+      if (tid == 0) p.out_count[slot] = 0;
+    }
     return;
   }
   const bool sampling = p.temperature > 0.f;
-  const int R = p.remaining[slot];
-  const int step = p.step[slot];
   int k = p.greedy_step ? 0 : min(p.K, R - 1);
   if (k < 0) k = 0;
   const int r0 = i * p.rps;
   const float *fq = p.forced_q ? p.forced_q + static_cast<size_t>(slot) * p.K * p.vocab : nullptr;
   // normalisers of the forced proposal distributions softmax(q / T)
   if (sampling && fq) {
-    for (int c = 0; c < k; ++c) {
+    for (int c = rank; c < k; c += C) {
       const float *row = fq + static_cast<size_t>(c) * p.vocab;
       float m = -INFINITY, sum = 0.f;
       for (int v = tid; v < p.vocab; v += kAccThreads) {
@@ -395,43 +454,54 @@ __global__ void __launch_bounds__(kAccThreads) accept_kernel(const AcceptParams 
         }
       }
       const float l = block_lse(m, sum, s_v, s_w);
-      if (tid == 0) s_qlse[c] = l;
+      if (tid < C) {
+        if (C > 1) dsmem_st_u32(dsmem_map(smem_u32(&s_qlse[c]), tid), __float_as_uint(l));
+        else s_qlse[c] = l;
+      }
     }
+    if (C > 1) cluster_sync();
+    else __syncthreads();
   }
+  // proposal c = tid + 1: accepted?
+  if (tid < k) {
+    const int c = tid + 1, cand = p.cand[slot * p.K + tid];
+    bool acc;
+    if (!sampling) {
+      acc = cand == p.tout[r0 + tid].arg;
+    } else {
+      const int rt = r0 + c - 1, rd = r0 + c;  // drafter row c holds mask position c
+      const float lse_t = p.tout[rt].lse;
+      const float lse_d = fq ? s_qlse[c - 1] : p.dout[rd].lse;
+      const float zd = fq ? fq[static_cast<size_t>(c - 1) * p.vocab + cand]
+                          : p.dlogits[static_cast<size_t>(rd) * p.vocab + cand];
+      const float xt = __fdiv_rn(p.tlogits[static_cast<size_t>(rt) * p.vocab + cand], p.temperature);
+      const float xd = __fdiv_rn(zd, p.temperature);
+      const bool sup = p.suppress && p.suppress[cand];
+      const float pc = sup ? 0.f : expf(xt - lse_t);
+      const float qc = sup ? 0.f : expf(xd - lse_d);
+      Philox4 o = philox4x32_10(0, c, step, (kTagAccept << 24) | (slot & 0xFFFFFF),
+                                static_cast<uint32_t>(p.seed), static_cast<uint32_t>(p.seed >> 32));
+      const float u = word_to_uniform(o.x[0]);
+      acc = u < __fdiv_rn(pc, qc);
+    }
+    s_cand[tid] = cand;
+    s_acc[tid] = acc;
+  }
+  __syncthreads();
   if (tid == 0) {
     int n_em = 0, a = 0, stop = 0, rej = 0;
     bool finished = false;
     for (int c = 1; c <= k; ++c) {
-      const int cand = p.cand[slot * p.K + c - 1];
-      bool acc;
-      if (!sampling) {
-        acc = cand == p.tout[r0 + c - 1].arg;
-      } else {
-        const int rt = r0 + c - 1, rd = r0 + c;  // drafter row c holds mask position c
-        const float lse_t = p.tout[rt].lse;
-        const float lse_d = fq ? s_qlse[c - 1] : p.dout[rd].lse;
-        const float zd = fq ? fq[static_cast<size_t>(c - 1) * p.vocab + cand]
-                            : p.dlogits[static_cast<size_t>(rd) * p.vocab + cand];
-        const float xt = __fdiv_rn(p.tlogits[static_cast<size_t>(rt) * p.vocab + cand], p.temperature);
-        const float xd = __fdiv_rn(zd, p.temperature);
-        const bool sup = p.suppress && p.suppress[cand];
-        const float pc = sup ? 0.f : expf(xt - lse_t);
-        const float qc = sup ? 0.f : expf(xd - lse_d);
-        Philox4 o = philox4x32_10(0, c, step, (kTagAccept << 24) | (slot & 0xFFFFFF),
-                                  static_cast<uint32_t>(p.seed), static_cast<uint32_t>(p.seed >> 32));
-        const float u = word_to_uniform(o.x[0]);
-        acc = u < __fdiv_rn(pc, qc);
-        if (!acc) {
-          rej = c;  // the residual draw below supplies the token
-          a = c - 1;
+      if (!s_acc[c - 1]) {
+        if (sampling) {  // the residual draw below supplies the token
+          rej = c;
           finished = true;
-          break;
         }
+        break;
       }
-      if (!acc) break;
-      s_em[n_em++] = cand;
+      s_em[n_em++] = s_cand[c - 1];
       a = c;
-      if (cand == p.eos) {
+      if (s_cand[c - 1] == p.eos) {
         stop = 1;
         finished = true;
         break;
@@ -459,45 +529,93 @@ __global__ void __launch_bounds__(kAccThreads) accept_kernel(const AcceptParams 
                          : p.dlogits + static_cast<size_t>(rd) * p.vocab;
     const float lse_t = p.tout[rt].lse;
     const float lse_d = fq ? s_qlse[rej - 1] : p.dout[rd].lse;
+    // this CTA's ids: whole groups of four (one Philox block each)
+    const int groups = (p.vocab + 3) / 4;
+    const int g0 = static_cast<int>(static_cast<long long>(groups) * rank / C);
+    const int g1 = static_cast<int>(static_cast<long long>(groups) * (rank + 1) / C);
+    const int warp = tid >> 5, lane = tid & 31;
     float best = -INFINITY;
     int barg = 0x7fffffff;
-    bool any = false;
-    for (int v = tid; v < p.vocab; v += kAccThreads) {
-      if (p.suppress && p.suppress[v]) continue;
-      const float pt = expf(__fdiv_rn(xt[v], p.temperature) - lse_t);
-      const float qd = expf(__fdiv_rn(xd[v], p.temperature) - lse_d);
-      const float r = fmaxf(pt - qd, 0.f);
-      if (r > 0.f) {
-        any = true;
-        const float sc = logf(r) + gumbel(p.seed, slot, step, rej, kTagResidual, v);
-        if (sc > best || (sc == best && v < barg)) {
-          best = sc;
-          barg = v;
+    // pass 0: the residual; pass 1 (if no CTA found any residual): the target
+    for (int pass = 0; pass < 2; ++pass) {
+      bool any = false;
+      float wbest = 0.f;  // the warp's best r / w so far
+      for (int gb = g0 + warp * 32; gb < g1; gb += kAccThreads) {
+        const int gq = gb + lane;
+        float rr[4], uu[4], est[4], top = 0.f;
+        const Philox4 o = philox4x32_10(static_cast<uint32_t>(gq), static_cast<uint32_t>(rej),
+                                        static_cast<uint32_t>(step), (kTagResidual << 24) | (slot & 0xFFFFFF),
+                                        static_cast<uint32_t>(p.seed), static_cast<uint32_t>(p.seed >> 32));
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int v = 4 * gq + e;
+          const bool live = gq < g1 && v < p.vocab && !(p.suppress && p.suppress[v]);
+          float r = live ? 1.f : 0.f;
+          if (live && pass == 0) {
+            const float pt = expf(__fdiv_rn(xt[v], p.temperature) - lse_t);
+            const float qd = expf(__fdiv_rn(xd[v], p.temperature) - lse_d);
+            r = fmaxf(pt - qd, 0.f);
+          }
+          rr[e] = r;
+          uu[e] = word_to_open_uniform(o.x[e]);
+          est[e] = __fdividef(r, neg_log2_estimate(uu[e]));
+          top = fmaxf(top, est[e]);
+        }
+        wbest = fmaxf(wbest, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top))));
+        // (the screen needs scores in the normal range; pass 1 scores all)
+        const float floor = pass == 0 && wbest > 1e-30f ? wbest - wbest * kRaceTol : 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (!(rr[e] > 0.f)) continue;
+          any = true;
+          if (est[e] < floor) continue;
+          const int v = 4 * gq + e;
+          const float x = pass == 0 ? logf(rr[e]) : __fdiv_rn(xt[v], p.temperature);
+          const float sc = x + -logf(-logf(uu[e]));
+          if (sc > best || (sc == best && v < barg)) {
+            best = sc;
+            barg = v;
+          }
         }
       }
-    }
-    if (!__syncthreads_or(any)) {
-      for (int v = tid; v < p.vocab; v += kAccThreads) {
-        if (p.suppress && p.suppress[v]) continue;
-        const float sc = __fdiv_rn(xt[v], p.temperature) + gumbel(p.seed, slot, step, rej, kTagResidual, v);
-        if (sc > best || (sc == best && v < barg)) {
-          best = sc;
-          barg = v;
+      any = __syncthreads_or(any);
+      block_argmax(best, barg, s_v, s_a);
+      if (C == 1) {
+        if (any) break;
+        continue;
+      }
+      // every CTA learns every CTA's best
+      if (tid < C) {
+        dsmem_st_u32(dsmem_map(smem_u32(&s_cv[rank]), tid), __float_as_uint(best));
+        dsmem_st_u32(dsmem_map(smem_u32(&s_ca[rank]), tid), any ? static_cast<uint32_t>(barg) : 0xffffffffu);
+      }
+      cluster_sync();
+      bool found = false;
+      best = -INFINITY;
+      barg = 0x7fffffff;
+      for (int q = 0; q < C; ++q) {
+        if (s_ca[q] < 0) continue;
+        found = true;
+        if (s_cv[q] > best || (s_cv[q] == best && s_ca[q] < barg)) {
+          best = s_cv[q];
+          barg = s_ca[q];
         }
       }
+      if (found) break;
+      cluster_sync();  // the exchange is read before the second pass rewrites it
     }
-    block_argmax(best, barg, s_v, s_a);
     if (tid == 0) {
       s_em[s_state[0]++] = barg;
       s_state[2] = barg == p.eos;
     }
   }
+  if (rank != 0) return;
   __syncthreads();
   const int n_em = s_state[0], a = s_state[1];
   for (int j = tid; j < Kp1; j += kAccThreads) p.out_tokens[slot * Kp1 + j] = j < n_em ? s_em[j] : -1;
   if (tid == 0) {
     p.out_count[slot] = n_em;
-    const int newL = p.L[slot] + 1 + a;
+    const int newL = L0 + 1 + a;
     p.L[slot] = newL;
     p.anchor[slot] = s_em[n_em - 1];
     const int left = R - n_em;
@@ -515,9 +633,25 @@ __global__ void __launch_bounds__(kAccThreads) accept_kernel(const AcceptParams 
 cudaError_t launch_accept(const AcceptParams &p0, cudaStream_t s, bool pdl) {
   AcceptParams p = p0;
   if (p.K > 8) return cudaErrorInvalidValue;
-  void *args[] = {&p};
-  return launch_ex(reinterpret_cast<const void *>(accept_kernel), dim3(p.n_seq > 0 ? p.n_seq : 1),
-                   dim3(kAccThreads), args, s, pdl);
+  const int n = p.n_seq > 0 ? p.n_seq : 1;
+  if (!(p.temperature > 0.f) || p.greedy_step) {
+    void *args[] = {&p};
+    return launch_ex(reinterpret_cast<const void *>(accept_kernel<1>), dim3(n), dim3(kAccThreads), args, s, pdl);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n * kAccCluster);
+  cfg.blockDim = dim3(kAccThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kAccCluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, accept_kernel<kAccCluster>, p);
 }
 
 // ---------------------------------------------------------------- state --
@@ -579,7 +713,8 @@ cudaError_t step_kernels_init() {
   static std::once_flag once;
   std::call_once(once, [] {
     const void *fns[] = {reinterpret_cast<const void *>(embed_kernel), reinterpret_cast<const void *>(layernorm_kernel),
-                         reinterpret_cast<const void *>(head_reduce_kernel), reinterpret_cast<const void *>(accept_kernel),
+                         reinterpret_cast<const void *>(head_reduce_kernel), reinterpret_cast<const void *>(accept_kernel<1>),
+                         reinterpret_cast<const void *>(accept_kernel<kAccCluster>),
                          reinterpret_cast<const void *>(state_kernel), reinterpret_cast<const void *>(compact_kernel)};
     status = cudaSuccess;
     for (const void *f : fns)
