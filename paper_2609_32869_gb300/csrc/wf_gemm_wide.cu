@@ -378,35 +378,67 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads<EPI>, 1
     int q = 0;
     pdl_wait();
     int par = 0, n_written = 0;
+    // The next tile's row table -- EPI_KV: (slot * heads * positions +
+    // position, 1), or (0, 0) past the cache; a sampling head: (slot and row of
+    // the block in the top byte, step) -- and its bias or masked ids, read while
+    // the current tile is worked on (their dependent loads cost 4500 cycles a
+    // tile in its path).
+    int2 next_tok = make_int2(0, 0);
+    bf16 next_b[4];
+    uint32_t next_masked = 0;
+    auto look_ahead = [&](int tile) {
+      if (tile >= tiles) return;
+      const int nt = tile / p.n_tt, n0 = (nt * 2 + rank) * 128, th = (tile - nt * p.n_tt) * BT + hg * gcols;
+      if constexpr (EPI == EPI_KV || EPI == EPI_HEAD) {
+        const int j = (ew & 3) * 32 + lane, t = th + j;
+        next_tok = make_int2(0, 0);
+        if (j < gcols && t < p.M && (EPI == EPI_KV || p.temperature > 0.f)) {
+          const int i = t / p.rows_per_seq, jr = t - i * p.rows_per_seq, slot = p.seq_slot[i];
+          if constexpr (EPI == EPI_KV) {
+            const int pos = (p.pos_base ? p.pos_base[slot] : 0) + jr;
+            if (pos < p.ctx) next_tok = make_int2(slot * p.n_heads * p.ctx + pos, 1);
+          } else {
+            next_tok = make_int2(slot | jr << 24, p.step[slot]);
+          }
+        }
+      }
+      next_masked = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int nn = n0 + 4 * lane + i;
+        if constexpr (EPI == EPI_HEAD) next_masked |= (nn >= p.N || (p.suppress && p.suppress[nn])) ? 1u << i : 0u;
+        else next_b[i] = (p.bias && nn < p.N) ? p.bias[nn] : __float2bfloat16(0.f);
+      }
+    };
+    look_ahead(pair);
     for (int tile = pair; tile < tiles; tile += n_pairs, par ^= 1) {
       const int ntile = (tile / p.n_tt) * 2 + rank, n0 = ntile * 128;
       const int th = (tile % p.n_tt) * BT + hg * gcols;  // first token row of the group
       int2 *tk = tok + par * 256 + hg * (256 / kGroups);
-      if constexpr (EPI == EPI_KV || EPI == EPI_HEAD) {
-        // (slot, position) of the group's rows, or for a sampling head (slot
-        // and row of the block in the top byte, step); the first slice's
-        // barrier publishes them
-        const int j = (ew & 3) * 32 + lane, t = th + j;
-        int2 sp = make_int2(0, 0x7fffffff);
-        if (j < gcols && t < p.M && (EPI == EPI_KV || p.temperature > 0.f)) {
-          const int i = t / p.rows_per_seq, jr = t - i * p.rows_per_seq;
-          sp.x = p.seq_slot[i];
-          if constexpr (EPI == EPI_KV) {
-            sp.y = (p.pos_base ? p.pos_base[sp.x] : 0) + jr;
-          } else {
-            sp.y = p.step[sp.x];
-            sp.x |= jr << 24;
-          }
-        }
-        if (j < gcols) tk[j] = sp;
-      }
+      // this tile's row table and bias were read under the previous tile; the
+      // first slice's barrier publishes the table
       float b4[4] = {0.f, 0.f, 0.f, 0.f};
       uint32_t masked = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int nn = n0 + 4 * lane + i;
-        if constexpr (EPI == EPI_HEAD) masked |= (nn >= p.N || (p.suppress && p.suppress[nn])) ? 1u << i : 0u;
-        else b4[i] = (p.bias && nn < p.N) ? bf2f(p.bias[nn]) : 0.f;
+        if constexpr (EPI == EPI_HEAD) masked = next_masked;
+        else b4[i] = bf2f(next_b[i]);
+      }
+      if constexpr (EPI == EPI_KV || EPI == EPI_HEAD) {
+        const int j = (ew & 3) * 32 + lane;
+        if (j < gcols) tk[j] = next_tok;
+      }
+      look_ahead(tile + n_pairs);
+      // EPI_KV: where this thread's four features go, from a row's table entry
+      bf16 *kv_q = nullptr, *kv_c = nullptr;
+      if constexpr (EPI == EPI_KV) {
+        const int n = n0 + 4 * lane;
+        if (n < p.q_cols) {
+          kv_q = p.out_bf16 + n;
+        } else if (n < p.N) {
+          const int c = n - p.q_cols, which = c / p.d_model, hd = c - which * p.d_model;
+          kv_c = (which == 0 ? p.kc : p.vc) + static_cast<size_t>(hd >> 6) * p.ctx * 64 + (hd & 63);
+        }
       }
       // the residual rows of a slice (this warp's four), loaded ahead of use
       float4 old[kR];
@@ -516,6 +548,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads<EPI>, 1
               const uint2 h = pack4_bf16(fin);
               if (p.tap0) *reinterpret_cast<uint2 *>(p.tap0 + static_cast<size_t>(t) * p.ld_tap + n0 + 4 * lane) = h;
               if (p.tap1) *reinterpret_cast<uint2 *>(p.tap1 + static_cast<size_t>(t) * p.ld_tap + n0 + 4 * lane) = h;
+            }
+          } else if constexpr (EPI == EPI_KV) {
+            if (valid) {
+              if (kv_q) {
+                *reinterpret_cast<uint2 *>(kv_q + static_cast<size_t>(t) * p.ld_out) = pack4_bf16(fin);
+              } else if (kv_c) {
+                const int2 at = tk[tl];
+                if (at.y) *reinterpret_cast<uint2 *>(kv_c + static_cast<size_t>(at.x) * 64) = pack4_bf16(fin);
+                else set_error(p.err, WF_DEV_ERR_CAPACITY);
+              }
             }
           } else if (valid) {
             float w4[4] = {v[0], v[1], v[2], v[3]};
