@@ -22,6 +22,7 @@
 // order.  Blocks and warps are aligned to absolute key positions and a key a
 // query cannot see contributes an exact zero, so a query's result does not
 // depend on how many other rows run with it.
+#include <cmath>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -899,32 +900,31 @@ __global__ void __launch_bounds__(kWkThreads, 2)
 
 // (cos, sin) of pos * base^(-2i/64) for every position below max_pos, or below
 // the last key of the call (n_seq > 0: the longest seq_slot / pos_base plus
-// rps).  The frequencies, one double-precision power each, are formed once per
-// CTA: double precision runs at 1/64 of the fp32 rate, and a power per entry
-// took 10 us at 448 positions.
-constexpr int kRopeRows = 16;  // positions per CTA
-__global__ void rope_table_kernel(float2 *tab, int max_pos, float base, const int32_t *seq_slot,
-                                  const int32_t *pos_base, int n_seq, int rps) {
-  __shared__ float s_inv[32];
-  if (threadIdx.x < 32) {
-    // inverse frequency base^(-2i/64) and the phase pos * inv_freq in FP32 (App. A.2)
-    const int i = threadIdx.x;
-    s_inv[i] = static_cast<float>(pow(static_cast<double>(base), -2.0 * i / 64.0));
-  }
-  __shared__ int s_rows;
-  if (threadIdx.x == 32) s_rows = n_seq > 0 ? 0 : max_pos;
-  __syncthreads();
-  for (int q = threadIdx.x; q < n_seq; q += blockDim.x) atomicMax(&s_rows, pos_base[seq_slot[q]] + rps);
-  __syncthreads();
-  const int rows = min(max_pos, s_rows);
-  for (int e = threadIdx.x; e < kRopeRows * 32; e += blockDim.x) {
-    const int pos = blockIdx.x * kRopeRows + e / 32, i = e % 32;
-    if (pos >= rows) continue;
-    const float ang = __fmul_rn(static_cast<float>(pos), s_inv[i]);
-    double sn, cs;
-    sincos(static_cast<double>(ang), &sn, &cs);
-    tab[pos * 32 + i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
-  }
+// rps).  Double precision runs at 2 operations per cycle and SM, and a sine and
+// cosine take ~100: the frequencies come from the host and two positions make
+// a CTA, so that the SMs share the rest (10.4 us at 159 positions with the
+// powers on the device and 16 positions a CTA).
+constexpr int kRopeRows = 2;  // positions per CTA
+struct RopeFreq {
+  float inv[32];  // base^(-2i/64), rounded from double
+};
+static RopeFreq rope_freq(float base) {
+  RopeFreq f;
+  for (int i = 0; i < 32; ++i) f.inv[i] = static_cast<float>(std::pow(static_cast<double>(base), -2.0 * i / 64.0));
+  return f;
+}
+__global__ void __launch_bounds__(32 * kRopeRows)
+    rope_table_kernel(float2 *tab, int max_pos, const RopeFreq f, const int32_t *seq_slot, const int32_t *pos_base,
+                      int n_seq, int rps) {
+  const int pos = blockIdx.x * kRopeRows + threadIdx.x / 32, i = threadIdx.x % 32;
+  bool used = n_seq == 0;
+  for (int q = i; q < n_seq; q += 32) used = used || pos < pos_base[seq_slot[q]] + rps;
+  if (!__any_sync(0xffffffffu, used) || pos >= max_pos) return;
+  // the phase pos * inv_freq in FP32 (App. A.2)
+  const float ang = __fmul_rn(static_cast<float>(pos), f.inv[i]);
+  double sn, cs;
+  sincos(static_cast<double>(ang), &sn, &cs);
+  tab[pos * 32 + i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
 }
 
 size_t attn_partial_floats(int n_seq, int rps, int n_heads, int ctx) {
@@ -1054,7 +1054,8 @@ cudaError_t launch_attention(const AttnParams &p0, cudaStream_t s, bool pdl) {
 }
 
 cudaError_t launch_rope_table(float2 *tab, int max_pos, float base, cudaStream_t s) {
-  rope_table_kernel<<<(max_pos + kRopeRows - 1) / kRopeRows, 256, 0, s>>>(tab, max_pos, base, nullptr, nullptr, 0, 0);
+  rope_table_kernel<<<(max_pos + kRopeRows - 1) / kRopeRows, 32 * kRopeRows, 0, s>>>(tab, max_pos, rope_freq(base), nullptr,
+                                                                                          nullptr, 0, 0);
   return cudaGetLastError();
 }
 
@@ -1088,8 +1089,8 @@ static wf_status attention_call(const void *d_q, const void *d_kc, const void *d
   if (rope) {
     float2 *tab = reinterpret_cast<float2 *>(static_cast<char *>(scratch) + pf * sizeof(float) +
                                              ((counters + 255) / 256) * 256);
-    rope_table_kernel<<<(ctx + kRopeRows - 1) / kRopeRows, 256, 0, s>>>(tab, ctx, rope_base, d_slot, d_base,
-                                                                       mode == 2 ? 0 : n_seq, RPS);
+    rope_table_kernel<<<(ctx + kRopeRows - 1) / kRopeRows, 32 * kRopeRows, 0, s>>>(tab, ctx, rope_freq(rope_base), d_slot,
+                                                                                      d_base, mode == 2 ? 0 : n_seq, RPS);
     if (cudaGetLastError() != cudaSuccess) return WF_ERR_CUDA;
     p.rope_tab = tab;
   }

@@ -125,14 +125,16 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_kernel(const __grid_cons
   uint4 *sZero = reinterpret_cast<uint4 *>(smem + L.zero_off);
   int *s_flag = reinterpret_cast<int *>(smem + L.flag_off);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int cta = blockIdx.x, split = blockIdx.z;
   const int unit0 = cta * U;  // first 8-row unit of this CTA
   const int n_base = unit0 * 8;
   const uint32_t crank = C > 1 ? cluster_ctarank() : 0u;  // cluster (C, 1, 1) when C > 1
 
   if (C > 1) cluster_arrive_relaxed();  // this CTA has started (peers write into it later)
-  if (tid == 0) {
+  // (barriers and copies by one elected lane of the first warp: under a thread
+  // comparison each copy took ~400 cycles to issue)
+  if (warp == 0 && elect_one()) {
     *s_flag = 0;
     tma_prefetch_desc(&tmW);
     if (tma_op) tma_prefetch_desc(&tmX);
@@ -208,7 +210,7 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_kernel(const __grid_cons
 
   // ---------------- operand: bf16 rows by one TMA copy (issued first), the
   // residual values this thread will update, or LN(x) shared by the cluster
-  if (tma_op && tid == 0) {
+  if (tma_op && warp == 0 && elect_one()) {
     mbar_arrive_expect_tx(&bar[1], static_cast<uint32_t>(L.a_bytes));
     tma_load_3d(sA, &tmX, 0, 0, split * kb, &bar[1]);
   }
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_xattn_kernel(const __gri
   uint4 *sZero = reinterpret_cast<uint4 *>(smem + L.zero_off);
   int *s_flag = reinterpret_cast<int *>(smem + L.flag_off);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int cta = blockIdx.x, head = cta >> 3;
   const uint32_t crank = cluster_ctarank();  // == cta % 8: this CTA's 8 dims of the head
   const int n_base = cta * 8;
@@ -586,7 +588,7 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_xattn_kernel(const __gri
   const long long spin = p.spin > 0 ? p.spin : kSpinLimitCycles;
 
   cluster_arrive_relaxed();  // this CTA has started (peers write into it later)
-  if (tid == 0) {
+  if (warp == 0 && elect_one()) {
     *s_flag = 0;
     tma_prefetch_desc(&tmW);
     tma_prefetch_desc(&tmX);
@@ -612,7 +614,7 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_xattn_kernel(const __gri
   pdl_wait();
 
   // ---------------- operand (rows g, b, then g . x) and the row statistics
-  if (tid == 0) {
+  if (warp == 0 && elect_one()) {
     mbar_arrive_expect_tx(&bar[1], static_cast<uint32_t>(kb * Mr * 128));
     tma_load_3d(sA, &tmX, 0, 0, 0, &bar[1]);
   }
@@ -951,7 +953,7 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_sattn_kernel(const __gri
   uint4 *sZero = reinterpret_cast<uint4 *>(smem + L.zero_off);
   int *s_flag = reinterpret_cast<int *>(smem + L.flag_off);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int cta = blockIdx.x, head = cta >> 3;
   const uint32_t crank = cluster_ctarank();
   const int nw = kpc / 32;
@@ -959,18 +961,8 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_sattn_kernel(const __gri
   const long long spin = p.spin > 0 ? p.spin : kSpinLimitCycles;
   // query, key and value units of this CTA (rows of the [3 d][d] weight)
   auto unit_row = [&](int u) { return (u * H * 8 + head * 8 + static_cast<int>(crank)) * 8; };
-  // the cache length and slot are fixed for the step (read before the wait)
-  const int slot = p.seq_slot[0];
-  const int Lc = p.pos_base[slot];
-  const int n_keys = Lc + M;
-  const bool fits = n_keys <= ctx;
-  const bool any_keys = fits && key0 < n_keys;
-  const int outer = slot * H + head;
-
   cluster_arrive_relaxed();  // this CTA has started (peers write into it later)
-  if (tid == 0) {
-    *s_flag = fits ? 0 : 1;
-    if (!fits) set_error(p.err, WF_DEV_ERR_CAPACITY);
+  if (warp == 0 && elect_one()) {  // the weights first: the cache's state is two loads away
     tma_prefetch_desc(&tmW);
     tma_prefetch_desc(&tmX);
     for (int i = 0; i < 4; ++i) mbar_init(&bar[i], 1);
@@ -978,6 +970,18 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_sattn_kernel(const __gri
     *sZero = make_uint4(0u, 0u, 0u, 0u);
     mbar_arrive_expect_tx(&bar[0], static_cast<uint32_t>(3 * kb * 1024));
     for (int u = 0; u < 3; ++u) tma_load_3d(sW + u * kb * 1024, &tmW, 0, unit_row(u), 0, &bar[0]);
+  }
+  __syncwarp();
+  // the cache length and slot are fixed for the step (read before the wait)
+  const int slot = p.seq_slot[0];
+  const int Lc = p.pos_base[slot];
+  const int n_keys = Lc + M;
+  const bool fits = n_keys <= ctx;
+  const bool any_keys = fits && key0 < n_keys;
+  const int outer = slot * H + head;
+  if (warp == 0 && elect_one()) {
+    *s_flag = fits ? 0 : 1;
+    if (!fits) set_error(p.err, WF_DEV_ERR_CAPACITY);
     if (any_keys) {  // this CTA's positions; rows from L on are replaced below
       tma_prefetch_desc(&tmK);
       tma_prefetch_desc(&tmV);
@@ -993,7 +997,7 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_sattn_kernel(const __gri
   pdl_wait();
 
   // ---------------- operand (rows g, b, then g . x) and the row statistics
-  if (tid == 0) {
+  if (warp == 0 && elect_one()) {
     mbar_arrive_expect_tx(&bar[1], static_cast<uint32_t>(kb * Mr * 128));
     tma_load_3d(sA, &tmX, 0, 0, 0, &bar[1]);
   }
