@@ -43,22 +43,19 @@ constexpr int kStageA = kBlockN * kBlockK * 2;  // 16 KB
 // Shared memory a CTA plans for: two CTAs fit on an SM, so one CTA's
 // epilogue overlaps the other's weight stream.
 constexpr int kSmemBudget = 110 * 1024;
-constexpr int kSmemBudgetLn = 110 * 1024;  // LN mode: resident token tiles + weight ring
 constexpr int kMaxBT = 128;                // token rows per tile (MMA N)
 constexpr size_t kSmemPerSM = 228 * 1024;  // shared memory of one SM
 constexpr uint32_t kGroupBytes = 128 * 4 * 4;  // one split's partials of four token rows
-// Token rows up to which LN is fused: every weight tile normalises the same
-// rows again, which at 144 rows costs 8-15 us per launch against a 4 us
-// LayerNorm kernel; at 32 rows the two forms are within 1%.
-constexpr int kLnFuseMaxM = 64;
 // Token rows above which pairs of SMs (wf_gemm_wide.cu) take a projection from
 // the cluster split-K.  Launches of a captured graph with weights from HBM, us
 // (cluster / pairs): 1280 x 1280 at 64, 96, 144 rows 6.3 / 7.8, 7.2 / 7.8,
 // 8.2 / 7.8; 1280 x 5120 9.8 / 13.9, 12.3 / 13.8, 15.6 / 13.9; 3840 x 1280 (30
 // weight tiles, so the pairs cover the GPU sooner) 7.7 / 7.5, 8.9 / 7.5,
-// 11.9 / 7.9; 5120 x 1280 8.2 / 7.7, 9.7 / 7.9, 12.9 / 8.4.
+// 11.9 / 7.9; 5120 x 1280 8.2 / 7.7, 9.7 / 7.9, 12.9 / 8.4.  A step of 6
+// sequences (54 rows) takes 529 us with its wide projections on clusters, 514
+// on pairs.
 constexpr int kWideMinM = 96;
-constexpr int kWideMinMFewRows = 64;
+constexpr int kWideMinMFewRows = 40;
 constexpr int kWideFewRowsN = 3840;
 
 // Epilogue of 16 consecutive token columns t0..t0+15 for output feature n.
@@ -123,73 +120,6 @@ __device__ __forceinline__ void epi_chunk(const GemmParams &p, int t0, int n, fl
   }
 }
 
-// Build the CTA's token operand for all kps k-steps from the fp32 residual:
-// B[i][r][k] = LN(x[t0 + r])[(kit0 + i) * 64 + k] as bf16, stored in the
-// 128-byte-swizzled K-major layout the TMA would have produced (16-byte
-// chunk j of row r at chunk position j ^ (r % 8)); rows past M are zero.
-__device__ __forceinline__ void ln_build_operand(const GemmParams &p, uint8_t *sB, uint32_t stageB,
-                                                 float2 *lnst, int t0, int kit0) {
-  const int BT = p.BT;
-  const int per_stage = BT * 8;
-  const int total = p.kps * per_stage;
-  constexpr int U = 4;
-  float4 xa[U], xb[U];
-  uint4 gv[U], bv[U];
-  // chunk c -> (k-step i, token row r, 16-byte chunk j of the 64-feature step)
-  auto load = [&](int c0) {
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int c = c0 + u * kThreads + static_cast<int>(threadIdx.x);
-      xa[u] = xb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      gv[u] = bv[u] = make_uint4(0u, 0u, 0u, 0u);
-      if (c < total) {
-        const int i = c / per_stage, rem = c - i * per_stage, r = rem >> 3, j = rem & 7;
-        const int t = t0 + r, f = (kit0 + i) * kBlockK + j * 8;
-        gv[u] = *reinterpret_cast<const uint4 *>(p.ln_g + f);
-        bv[u] = *reinterpret_cast<const uint4 *>(p.ln_b + f);
-        if (t < p.M) {
-          const float4 *src =
-              reinterpret_cast<const float4 *>(p.ln_x + static_cast<size_t>(t) * p.ln_ld + f);
-          xa[u] = src[0];
-          xb[u] = src[1];
-        }
-      }
-    }
-  };
-  load(0);  // the first rows are in flight while the statistics merge
-  for (int j = threadIdx.x; j < BT; j += blockDim.x) {
-    const int t = t0 + j;
-    lnst[j] = t < p.M ? merge_tile_stats(p.ln_stats + static_cast<size_t>(t) * p.ln_tiles,
-                                         p.ln_tiles, p.ln_eps)
-                      : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  for (int c0 = 0; c0 < total; c0 += U * kThreads) {
-    if (c0) load(c0);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int c = c0 + u * kThreads + static_cast<int>(threadIdx.x);
-      if (c >= total) continue;
-      const int i = c / per_stage, rem = c - i * per_stage, r = rem >> 3, j = rem & 7;
-      uint4 o = make_uint4(0u, 0u, 0u, 0u);
-      if (t0 + r < p.M) {
-        const float2 ms = lnst[r];
-        const __nv_bfloat162 *g2 = reinterpret_cast<const __nv_bfloat162 *>(&gv[u]);
-        const __nv_bfloat162 *b2 = reinterpret_cast<const __nv_bfloat162 *>(&bv[u]);
-        const float xs[8] = {xa[u].x, xa[u].y, xa[u].z, xa[u].w, xb[u].x, xb[u].y, xb[u].z, xb[u].w};
-        __nv_bfloat162 h[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          h[q] = __floats2bfloat162_rn(
-              ln_apply(xs[2 * q], ms, __low2float(g2[q]), __low2float(b2[q])),
-              ln_apply(xs[2 * q + 1], ms, __high2float(g2[q]), __high2float(b2[q])));
-        o = *reinterpret_cast<const uint4 *>(h);
-      }
-      *reinterpret_cast<uint4 *>(sB + static_cast<size_t>(i) * stageB + r * 128 + ((j ^ (r & 7)) << 4)) = o;
-    }
-  }
-}
-
 template <int EPI>
 __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW,
                                                       const __grid_constant__ CUtensorMap tmX,
@@ -208,11 +138,9 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 2);
   // per-token (slot, position) for EPI_KV, (slot, step) for sampling heads
   int2 *tok = reinterpret_cast<int2 *>(smem + p.pipe_bytes + (2 * stages + 2) * 8 + 32);
-  float2 *lnst = reinterpret_cast<float2 *>(tok + BT);  // per-token (mean, rstd), LN mode
   // split-K: where the partials of each group of four token rows go (the
   // cluster addresses of the slot and of its owner's inbox barrier)
-  uint2 *dest = reinterpret_cast<uint2 *>(lnst + (p.ln_x ? BT : 0));
-  const bool ln = p.ln_x != nullptr;
+  uint2 *dest = reinterpret_cast<uint2 *>(tok + BT);
   // a bounded wait of this CTA gave up (in the 32 bytes reserved after the
   // barriers, beside the TMEM address; the kernel has no static shared memory)
   volatile int &s_timed_out = *reinterpret_cast<int *>(tmem_slot + 1);
@@ -243,12 +171,11 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   pdl_launch_dependents();
 
   // Weight tiles of the first stages do not depend on the previous kernel:
-  // request them before the dependency wait.  In LN mode each stage carries
-  // only its weight tile; the token operand is built once for all k-steps.
+  // request them before the dependency wait.
   // Copies and MMAs are issued by one elected lane of code that the whole warp
   // runs: under a lane comparison each of them took ~430 cycles.
   const int npre = kps < stages ? kps : stages;
-  const uint32_t tx = ln ? static_cast<uint32_t>(kStageA) : kStageA + stageB;
+  const uint32_t tx = kStageA + stageB;
   if (warp == 0) {
     for (int i = 0; i < npre; ++i) {
       if (elect_one()) {
@@ -257,22 +184,12 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
       }
     }
   }
-  if (ln) {
-    pdl_wait();  // the residual rows and their statistics come from the previous kernels
-    ln_build_operand(p, sB, stageB, lnst, t0, kit0);
-    fence_proxy_async();  // generic-proxy writes -> visible to tcgen05.mma
-    __syncthreads();
-  }
-
   int issued = npre;  // k-steps whose tiles the producer (warp 0) has requested
   if (warp == 0) {
     // ---------------- TMA producer
-    if (!ln) {
-      pdl_wait();  // token rows come from the previous kernel
-      for (int i = 0; i < npre; ++i)
-        if (elect_one())
-          tma_load_2d(sB + static_cast<size_t>(i) * stageB, &tmX, (kit0 + i) * kBlockK, t0, &full[i]);
-    }
+    pdl_wait();  // token rows come from the previous kernel
+    for (int i = 0; i < npre; ++i)
+      if (elect_one()) tma_load_2d(sB + static_cast<size_t>(i) * stageB, &tmX, (kit0 + i) * kBlockK, t0, &full[i]);
     int s = 0;
     uint32_t ph = 0;
     for (int it = npre; it < kps; ++it) {  // (only when npre == stages)
@@ -284,8 +201,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
       if (elect_one()) {
         mbar_arrive_expect_tx(&full[s], tx);
         tma_load_2d(sA + static_cast<size_t>(s) * kStageA, &tmW, (kit0 + it) * kBlockK, n0, &full[s]);
-        if (!ln)
-          tma_load_2d(sB + static_cast<size_t>(s) * stageB, &tmX, (kit0 + it) * kBlockK, t0, &full[s]);
+        tma_load_2d(sB + static_cast<size_t>(s) * stageB, &tmX, (kit0 + it) * kBlockK, t0, &full[s]);
       }
       if (++s == stages) {
         s = 0;
@@ -308,7 +224,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
       tc_fence_after();
       if (elect_one()) {
         const uint64_t ad = a_base + static_cast<uint64_t>((s * kStageA) >> 4);
-        const uint64_t bd = b_base + static_cast<uint64_t>(((ln ? it : s) * stageB) >> 4);
+        const uint64_t bd = b_base + static_cast<uint64_t>((s * stageB) >> 4);
 #pragma unroll
         for (int kk = 0; kk < kBlockK / 16; ++kk)
           umma_bf16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (it | kk) != 0 ? 1u : 0u);
@@ -710,32 +626,17 @@ static bool plan_gemm(GemmParams &p, size_t *smem_out) {
   const int k_iters = p.K / kBlockK;
   if (k_iters % p.splits) return false;
   p.kps = k_iters / p.splits;
-  const bool ln = p.ln_x != nullptr;
   const size_t stageA = kStageA, stageB = static_cast<size_t>(p.BT) * kBlockK * 2;
-  const size_t red = static_cast<size_t>(p.BT) * sizeof(int2) * (ln ? 2 : 1) +
+  const size_t red = static_cast<size_t>(p.BT) * sizeof(int2) +
                      (p.splits > 1 ? static_cast<size_t>(p.BT / 4) * sizeof(uint2) : 0);
-  const size_t fixed = red;
   uint32_t cols = 32;
   while (cols < static_cast<uint32_t>(p.BT)) cols <<= 1;
   p.tmem_cols = cols;
-  const size_t budget = kSmemBudget;
-  int stages;
-  size_t pipe;
-  if (ln) {
-    // every k-step's token tile stays resident; the weight tiles cycle through a ring
-    const size_t btiles = static_cast<size_t>(p.kps) * stageB;
-    if (btiles + 2 * stageA + fixed > kSmemBudgetLn) return false;
-    stages = static_cast<int>((kSmemBudgetLn - fixed - btiles) / stageA);
-    if (stages > p.kps) stages = p.kps;
-    if (stages > 16) stages = 16;
-    pipe = stages * stageA + btiles;
-  } else {
-    if (fixed + stageA + stageB > budget) return false;
-    stages = static_cast<int>((budget - fixed) / (stageA + stageB));
-    if (stages > p.kps) stages = p.kps;
-    if (stages > 16) stages = 16;
-    pipe = stages * (stageA + stageB);
-  }
+  if (red + stageA + stageB > kSmemBudget) return false;
+  int stages = static_cast<int>((kSmemBudget - red) / (stageA + stageB));
+  if (stages > p.kps) stages = p.kps;
+  if (stages > 16) stages = 16;
+  size_t pipe = stages * (stageA + stageB);
   p.stages = stages;
   // the staged epilogues reuse the pipeline buffers for a [BT][128] fp32 tile
   if (p.stats_out) pipe = std::max<size_t>(pipe, 512 * static_cast<size_t>(p.BT));
@@ -754,52 +655,27 @@ static bool plan_gemm(GemmParams &p, size_t *smem_out) {
   return true;
 }
 
-bool gemm_ln_fits(int M, int N, int K, int epi) {
-  // Every weight tile of the projection normalises the same token rows again;
-  // past one token tile that repeated work outweighs the launch it saves.
-  if (M > kLnFuseMaxM) return false;
-  GemmParams p = {};
-  p.M = M;
-  p.N = N;
-  p.K = K;
-  p.epi = epi;
-  p.splits = gemm_splits(N, K);
-  p.ln_x = reinterpret_cast<const float *>(16);  // only tested for non-null
-  size_t smem = 0;
-  return plan_gemm(p, &smem);
-}
-
 cudaError_t launch_gemm(const void *X, const void *W, GemmParams p, cudaStream_t s, bool pdl) {
-  const bool ln = p.ln_x != nullptr;
   if (p.spin <= 0) p.spin = kSpinLimitCycles;
   const bool quad = p.splits > 1 || p.stats_out;  // the staged (four-feature) epilogue
-  if (p.epi == EPI_HEAD && (ln || p.stats_out)) return cudaErrorInvalidValue;
+  if (!X || (p.epi == EPI_HEAD && p.stats_out)) return cudaErrorInvalidValue;
   if ((p.stats_out || p.epi == EPI_RESID) && p.N % kBlockN) return cudaErrorInvalidValue;
   if (p.epi == EPI_RESID && (p.ld_resid % 4 || (reinterpret_cast<uintptr_t>(p.resid) & 15)))
     return cudaErrorInvalidValue;
   if (quad && p.epi == EPI_KV && (p.N % 4 || p.q_cols % 4 || p.d_model % 4 || p.ld_out % 4))
     return cudaErrorInvalidValue;
   if (quad && p.epi == EPI_RESID && (p.tap0 || p.tap1) && p.ld_tap % 4) return cudaErrorInvalidValue;
-  if (ln) {
-    const uintptr_t al = reinterpret_cast<uintptr_t>(p.ln_x) | reinterpret_cast<uintptr_t>(p.ln_g) |
-                         reinterpret_cast<uintptr_t>(p.ln_b);
-    if (!p.ln_stats || !p.ln_g || !p.ln_b || (al & 15) || p.ln_ld % 4 || p.ln_tiles < 1 || p.ln_tiles > kMaxStatTiles ||
-        p.K > p.ln_tiles * 128 || p.ln_ld < p.K)
-      return cudaErrorInvalidValue;
-  } else if (!X) {
-    return cudaErrorInvalidValue;
-  }
   // Past kWideMinM rows pairs of SMs on 256-row weight tiles (same bits).
   // They write four features at a time whatever the split, so a key/value
   // scatter with odd strides stays here.  They run the output head at any
   // number of rows.
   const bool quads = p.epi != EPI_KV || !(p.N % 4 || p.q_cols % 4 || p.d_model % 4 || p.ld_out % 4);
   const int wide_m = p.N >= kWideFewRowsN ? kWideMinMFewRows : kWideMinM;
-  if (p.epi == EPI_HEAD || (!ln && p.M > wide_m && quads)) return launch_gemm_wide(X, W, p, s, pdl);
+  if (p.epi == EPI_HEAD || (p.M > wide_m && quads)) return launch_gemm_wide(X, W, p, s, pdl);
   size_t smem = 0;
   if (!plan_gemm(p, &smem)) return cudaErrorInvalidValue;
   const CUtensorMap *tw = tmap_bf16_2d(W, p.N, p.K, kBlockN);
-  const CUtensorMap *tx = ln ? tw : tmap_bf16_2d(X, p.M, p.K, p.BT);
+  const CUtensorMap *tx = tmap_bf16_2d(X, p.M, p.K, p.BT);
   if (!tw || !tx) return cudaErrorInvalidValue;
   switch (p.epi) {
     case EPI_F32: return launch_typed<EPI_F32>(tw, tx, p, smem, s, pdl);

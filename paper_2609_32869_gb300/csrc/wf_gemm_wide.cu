@@ -163,8 +163,8 @@ __device__ __forceinline__ void head_rows_sample(const GemmParams &p, const floa
   }
   // Exact scores of the candidates: each lane's first one of every row
   // together, further ones (rare) after.
-  uint32_t cand[R], gkey[R];
-  int gid[R];
+  uint32_t cand[R] = {}, gkey[R] = {};
+  int gid[R] = {};
   auto take = [&](int k) {  // score row k's lowest candidate of this lane
     const int i = __ffs(static_cast<int>(cand[k])) - 1;
     const float zi = i == 0 ? z[k][0] : i == 1 ? z[k][1] : i == 2 ? z[k][2] : z[k][3];
@@ -652,7 +652,7 @@ static cudaError_t gemm_wide_init() {
 // Token tile, ring depth and grid of a launch; false if the kernel does not
 // take the shape.
 static bool gemm_wide_plan(GemmParams &p, size_t *smem, int *pairs) {
-  if (p.M <= 0 || p.N <= 0 || p.K <= 0 || p.K % 64 || p.ln_x) return false;
+  if (p.M <= 0 || p.N <= 0 || p.K <= 0 || p.K % 64) return false;
   if (p.splits < 1 || p.epi == EPI_HEAD) p.splits = 1;
   const int k_iters = p.K / 64;
   if (k_iters % p.splits) return false;

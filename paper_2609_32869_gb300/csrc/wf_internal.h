@@ -78,15 +78,6 @@ struct GemmParams {
   uint32_t tag;
   uint32_t *err;
   long long spin;  // clock cycles a bounded wait spins before it gives up
-  // LayerNorm-fused token operand: when ln_x is set the CTA builds its bf16
-  // B tiles as LN(x) = (x - mean) * rstd * g + b from fp32 rows ln_x (row
-  // stride ln_ld) and per-row statistics ln_stats[t][0..ln_tiles) (mean, M2
-  // over each 128-feature tile, merged in tile order); X is then unused.
-  const float *ln_x;
-  int ln_ld, ln_tiles;
-  const float2 *ln_stats;
-  const bf16 *ln_g, *ln_b;
-  float ln_eps;
   // Statistics of this GEMM's outputs for the next LayerNorm: per output row
   // and 128-feature tile, (mean, M2) of the final values (the updated
   // residual for EPI_RESID, the output for EPI_F32); [M][N/128].
@@ -112,16 +103,10 @@ int gemm_splits(int N, int K);
 
 // Opt every GEMM instantiation into large dynamic shared memory (once).
 cudaError_t gemm_init();
-// Launch one GEMM.  W is [N, K] bf16, X is [M, K] bf16 (row stride K), or
-// X is null and the token operand is LN(p.ln_x) built inside the kernel.
+// Launch one GEMM.  W is [N, K] bf16, X is [M, K] bf16 (row stride K).
 cudaError_t launch_gemm(const void *X, const void *W, GemmParams p, cudaStream_t s, bool pdl);
-// Whether to use the LayerNorm-fused form of a launch: one token tile, and
-// all of the CTA's token tiles fit in shared memory; otherwise run
-// launch_layernorm first (same bits either way).
-bool gemm_ln_fits(int M, int N, int K, int epi);
-
 // The same projections for many token rows on pairs of SMs (wf_gemm_wide.cu);
-// same arguments and bits as launch_gemm, no LayerNorm-fused operand.
+// same arguments and bits as launch_gemm.
 cudaError_t launch_gemm_wide(const void *X, const void *W, GemmParams p, cudaStream_t s, bool pdl);
 
 // ------------------------------------------------------ skinny projections --
