@@ -85,13 +85,13 @@ GEMM_DRAM_BYTES_PER_LAUNCH = {
     # 68 x out/cross-out (3.404 MB), 34 x fc1 (13.219), 34 x fc2 (13.313),
     # 2 x history K/V (6.662), 1 x history projection (16.572) per step
     "large_b1": 8.370e6,
-    # 34 x QKV (12.077 MB), 102 x out/cross-out/fc2 (15.296), 34 x cross-query
-    # (5.514), 34 x fc1 (15.354), 2 x history K/V (8.796), 1 x history
-    # projection (27.283) per step, captured at 94 sequences
-    "large_b96": 13.165e6,
+    # 34 x QKV (12.064 MB), 102 x out/cross-out/fc2 (15.277), 34 x cross-query
+    # (5.507), 34 x fc1 (15.361), 2 x history K/V (8.781), 1 x history
+    # projection (27.277) per step, captured at 94 sequences
+    "large_b96": 13.154e6,
     # 204 x batched skinny projections (8.593 MB), 2 x history K/V (7.346), 1 x
     # history projection (18.194) per step, captured at 15 live sequences with
-    # --skinny (the default batch-16 path is tcgen05, which no capture covers)
+    # --skinny (the default path, tcgen05, moves 8.608 MB per launch there)
     "large_b16": 8.627e6,
 }
 
@@ -107,7 +107,7 @@ def _proj_kernel(path, rows):
     """The kernel that runs a pass's projections: the skinny kernels up to 144
     step rows (one operand tile up to 14), else the tcgen05 GEMM."""
     if path != "skinny":
-        return "gemm_tc_kernel (tcgen05 projections)"
+        return "gemm_tc_kernel / gemm_wide_kernel (tcgen05 projections)"
     if rows <= 14:
         return "skinny_kernel (single-sequence projections)"
     return "skinny_mt_kernel (batched skinny projections)"
@@ -116,9 +116,9 @@ def _proj_kernel(path, rows):
 # Tensor-pipe activity of the projections at batch 96 from the committed ncu
 # capture of the same kernels (profiles/), or absent until one is taken.
 TENSOR_PIPE_FROM_PROFILE = {
-    "large_b96": {"pct_of_peak_elapsed_time_weighted": 7.8,
-                  "by_projection": {"fc1": 12.0, "QKV": 9.1, "cross_query": 6.2,
-                                    "out_crossout_fc2": 5.7, "history_kv": 10.1},
+    "large_b96": {"pct_of_peak_elapsed_time_weighted": 16.9,
+                  "by_projection": {"fc1": 20.5, "QKV": 18.7, "cross_query": 9.7,
+                                    "out_crossout_fc2": 15.0, "history_kv": 17.1},
                   "source": "profiles/dram_per_kernel_large_b96_2l.md (ncu, 94 sequences, 2 target blocks)"},
 }
 

@@ -251,7 +251,7 @@ int32_t wf_last_launch_count(const wf_handle *h);
                                 resident, more with it streamed by k-block); 0: the tcgen05
                                 projections.  Default 1 when max_batch * (block_k + 1) <= 14
                                 (single-sequence handles), else 0 (the streamed form is
-                                slower than tcgen05 at 2-8 sequences and ties it at 16).
+                                slower than the tcgen05 projections).
                                 Setting 1 on a handle of more than 144 step rows returns
                                 WF_ERR_UNSUPPORTED.
                                 The two forms agree within the method's tolerances, not bit

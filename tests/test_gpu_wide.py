@@ -31,8 +31,8 @@ def test_wide_rows_equal_small_launches(N, K):
         B.wf_gemm_bf16(x[lo:hi], w, b, y, hi - lo, N, K, None, 0)
         return y
 
-    want = torch.cat([run(lo, min(M, lo + 60)) for lo in range(0, M, 60)])  # cluster split-K
-    for m in (65, 96, 97, 129, 257, 288, 833, M):
+    want = torch.cat([run(lo, min(M, lo + 40)) for lo in range(0, M, 40)])  # cluster split-K
+    for m in (41, 65, 96, 97, 129, 257, 288, 833, M):
         assert torch.equal(run(0, m), want[:m]), m
     assert torch.equal(run(0, 300, offset=1), want[:300])  # an output that is only 4-byte aligned
     bound = K * 2.0 ** -23 * (x.double().abs() @ w.double().abs().T) + 1e-6
