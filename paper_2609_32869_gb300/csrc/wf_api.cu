@@ -1064,8 +1064,8 @@ wf_status wf_create(const wf_config *cfg, const wf_target_weights *tw, const wf_
   h->sk_rows = max_batch * (cfg->block_k + 1);
   h->skinny_ok = skinny_shapes_fit(h->d, h->F, h->sk_rows);
   // on by default where one operand tile holds a pass (single-sequence
-  // handles); the batched form (2-16 sequences) is opt-in: it measured 3-12%
-  // slower per step than the tcgen05 projections at 2-8 sequences, a tie at 16
+  // handles); the batched form (2-16 sequences) is opt-in: a step of 16
+  // sequences takes 4.25 ms with it, 3.48 with the tcgen05 projections
   h->skinny = h->skinny_ok && h->sk_rows <= kSkMaxFoldRows;
   ok = ok && gemm_init() == cudaSuccess && skinny_init() == cudaSuccess && skinny_mt_init() == cudaSuccess &&
        attention_init() == cudaSuccess &&
