@@ -979,12 +979,13 @@ cudaError_t attention_init() {
 // leaving the same partials and merging them itself (a single wave of CTAs, no
 // counter), or, over the acoustic memory, where every group has as many
 // blocks, persistent CTAs walk even shares of all blocks (cross_walk_kernel,
-// with its measurements).  All do the same arithmetic in the same order.
+// with its measurements; it does not rotate, so a call with a RoPE table stays
+// with one CTA per group).  All do the same arithmetic in the same order.
 struct AttnForm {
   int n_sm, qgroups, n_chunks, cluster, loop, walk;
   bool counters() const { return n_chunks > 1 && !cluster && !loop; }  // the form counts finished blocks
 };
-static AttnForm attn_form(int n_seq, int rps, int n_heads, int ctx, int mode) {
+static AttnForm attn_form(int n_seq, int rps, int n_heads, int ctx, int mode, bool rope) {
   static const int n_sm = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -999,14 +1000,14 @@ static AttnForm attn_form(int n_seq, int rps, int n_heads, int ctx, int mode) {
   const long long groups = static_cast<long long>(n_seq) * n_heads * f.qgroups;
   f.cluster = (f.n_chunks > 1 && f.n_chunks <= 8 && groups * f.n_chunks <= n_sm) ? 1 : 0;
   const bool many = !f.cluster && f.n_chunks > 1 && n_sm > 0 && groups >= 2LL * n_sm;
-  f.walk = (many && mode == 2 && groups * f.n_chunks <= 0x3fffffff) ? 1 : 0;
+  f.walk = (many && mode == 2 && !rope && groups * f.n_chunks <= 0x3fffffff) ? 1 : 0;
   f.loop = (many && !f.walk) ? 1 : 0;
   return f;
 }
 
 cudaError_t launch_attention(const AttnParams &p0, cudaStream_t s, bool pdl) {
   AttnParams p = p0;
-  AttnForm f = attn_form(p.n_seq, p.rps, p.n_heads, p.ctx, p.mode);
+  AttnForm f = attn_form(p.n_seq, p.rps, p.n_heads, p.ctx, p.mode, p.rope_tab != nullptr);
   if (f.walk && (reinterpret_cast<uintptr_t>(p.part) & 7)) {  // its partials go out in pairs
     f.walk = 0;
     f.loop = 1;
@@ -1084,7 +1085,8 @@ static wf_status attention_call(const void *d_q, const void *d_kc, const void *d
   const size_t counters = static_cast<size_t>(attn_counter_slots(n_seq, RPS, n_heads)) * 4;
   p.part = static_cast<float *>(scratch);
   p.counters = reinterpret_cast<int32_t *>(static_cast<char *>(scratch) + pf * sizeof(float));
-  if (attn_form(n_seq, RPS, n_heads, ctx, mode).counters() && cudaMemsetAsync(p.counters, 0, counters, s) != cudaSuccess)
+  if (attn_form(n_seq, RPS, n_heads, ctx, mode, rope != 0).counters() &&
+      cudaMemsetAsync(p.counters, 0, counters, s) != cudaSuccess)
     return WF_ERR_CUDA;
   if (rope) {
     float2 *tab = reinterpret_cast<float2 *>(static_cast<char *>(scratch) + pf * sizeof(float) +
