@@ -781,11 +781,13 @@ __global__ void __launch_bounds__(kWkThreads, 2)
         mrow[r] = fmaxf(mrow[r], __shfl_xor_sync(0xffffffffu, mrow[r], 1));
         mrow[r] = fmaxf(mrow[r], __shfl_xor_sync(0xffffffffu, mrow[r], 2));
       }
+      // (a row whose scores here are all -inf has no maximum: weights 0, not NaN)
+      const float mfin[2] = {mrow[0] == -INFINITY ? 0.f : mrow[0], mrow[1] == -INFINITY ? 0.f : mrow[1]};
 #pragma unroll
       for (int nt = 0; nt < kNT; ++nt)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float v = exp2f_fast(s[nt][e] - mrow[e >> 1]);
+          const float v = exp2f_fast(s[nt][e] - mfin[e >> 1]);
           s[nt][e] = v;
           lrow[e >> 1] += v;
         }
@@ -853,16 +855,17 @@ __global__ void __launch_bounds__(kWkThreads, 2)
         mw[v] = sm[v * kQG + qi];
         M = fmaxf(M, mw[v]);
       }
+      const float mf = M == -INFINITY ? 0.f : M;
 #pragma unroll
       for (int v = 0; v < kWarps; ++v) {
-        const float wt = exp2f_fast(mw[v] - M);  // (0 for -inf)
+        const float wt = exp2f_fast(mw[v] - mf);  // (0 for -inf)
         const float4 o4 = *reinterpret_cast<const float4 *>(so + (v * kQG + qi) * 64 + (d0 ^ ((qi & 3) << 3)));
         L = __fmaf_rn(sl[v * kQG + qi], wt, L);
-        // (a slice without a key left its O unwritten)
-        acc[0] = wt == 0.f ? acc[0] : __fmaf_rn(o4.x, wt, acc[0]);
-        acc[1] = wt == 0.f ? acc[1] : __fmaf_rn(o4.y, wt, acc[1]);
-        acc[2] = wt == 0.f ? acc[2] : __fmaf_rn(o4.z, wt, acc[2]);
-        acc[3] = wt == 0.f ? acc[3] : __fmaf_rn(o4.w, wt, acc[3]);
+        const bool none = mw[v] == -INFINITY;  // (a slice without a key left its O unwritten)
+        acc[0] = none ? acc[0] : __fmaf_rn(o4.x, wt, acc[0]);
+        acc[1] = none ? acc[1] : __fmaf_rn(o4.y, wt, acc[1]);
+        acc[2] = none ? acc[2] : __fmaf_rn(o4.z, wt, acc[2]);
+        acc[3] = none ? acc[3] : __fmaf_rn(o4.w, wt, acc[3]);
       }
     }
     fence_proxy_async();  // the tile's generic writes and reads come before its next copy

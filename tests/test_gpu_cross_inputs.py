@@ -1,5 +1,6 @@
 """Cross-attention of many sequences on the inputs that its entry point takes
-besides plain queries and keys: rotated by position (`rope`).  A large launch equals launches of its sequences alone,
+besides plain queries and keys: rotated by position (`rope`), and with frames
+whose scores are -inf.  A large launch equals launches of its sequences alone,
 bit for bit, and the oracle."""
 import numpy as np
 import pytest
@@ -9,7 +10,7 @@ from oracle import decoder as od
 pytestmark = pytest.mark.gpu
 
 
-def _calls(n_seq, rps, H, ctx, rope):
+def _calls(n_seq, rps, H, ctx, rope, edit=None):
     """(rows per sequence of one launch, of one launch each, of the oracle)."""
     import torch
     from paper_2609_32869_gb300 import binding as B
@@ -19,6 +20,8 @@ def _calls(n_seq, rps, H, ctx, rope):
     q = torch.randn(n_seq * rps, d, generator=g, device="cuda").bfloat16()
     k = torch.randn(n_seq, H, ctx, 64, generator=g, device="cuda").bfloat16()
     v = torch.randn(n_seq, H, ctx, 64, generator=g, device="cuda").bfloat16()
+    if edit:
+        edit(q.view(n_seq * rps, H, 64), k)
 
     def run(rows, sl, noalloc=False):
         n = len(sl)
@@ -58,4 +61,23 @@ def test_positions_rotate_whatever_the_number_of_sequences(n_seq, rps, H, ctx):
     big, alone, ends, want = _calls(n_seq, rps, H, ctx, 1)
     assert torch.equal(big, alone)
     # bf16 output rounding (2^-8 relative) dominates the fp32 arithmetic
+    np.testing.assert_allclose(ends, want, atol=2e-2, rtol=1e-2)
+
+
+# frames whose keys are -inf against positive queries: slices of 32 keys, a
+# whole block of 256, the cut last block, and all but one frame
+@pytest.mark.parametrize("n_seq,rps,H,ctx,masked", [
+    (17, 9, 20, 600, ((64, 128),)), (17, 9, 20, 600, ((0, 33), (256, 512))), (17, 9, 20, 600, ((512, 600),)),
+    (9, 17, 20, 513, ((0, 256), (288, 513))), (53, 9, 6, 300, ((0, 299),)), (15, 9, 20, 600, ((64, 128), (256, 512)))])
+def test_masked_frames_have_weight_zero(n_seq, rps, H, ctx, masked):
+    import torch
+
+    def edit(q, k):
+        q[..., 0] = 1.0
+        for a, b in masked:
+            k[:, :, a:b, 0] = float("-inf")
+
+    big, alone, ends, want = _calls(n_seq, rps, H, ctx, 0, edit)
+    assert torch.isfinite(big.float()).all()
+    assert torch.equal(big, alone)
     np.testing.assert_allclose(ends, want, atol=2e-2, rtol=1e-2)
