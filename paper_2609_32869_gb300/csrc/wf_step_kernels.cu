@@ -468,6 +468,10 @@ __global__ void __launch_bounds__(kAccThreads) accept_kernel(const AcceptParams 
     bool acc;
     if (!sampling) {
       acc = cand == p.tout[r0 + tid].arg;
+    } else if (cand < 0 || cand >= p.vocab) {
+      // no such id (the embedding has recorded it): probability 0, so rejected.
+      // All proposals are looked at together, also those behind a rejection.
+      acc = false;
     } else {
       const int rt = r0 + c - 1, rd = r0 + c;  // drafter row c holds mask position c
       const float lse_t = p.tout[rt].lse;
