@@ -374,7 +374,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads<EPI>, 1
     const int feat = quarter * 32 + lane;  // this thread's feature of the 128
     float *buf0 = stg + hg * 2 * kSlice * 128;
     const int stat_tiles = p.N / 128;
-    bool ok = true;
+    bool ok = true;  // the same in all lanes: the head's reductions take the whole warp
     int q = 0;
     pdl_wait();
     int par = 0, n_written = 0;
@@ -458,7 +458,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads<EPI>, 1
       if constexpr (HC > 0) {
         // add the chunks in order from zero, two 16-column loads in flight
         for (int r = 0; r < p.splits; ++r, ++q) {
-          if (ok && !mbar_wait(&accf[q & 1], static_cast<uint32_t>(q >> 1) & 1u, p.err, p.spin)) ok = false;
+          if (ok) ok = warp_mbar_wait(&accf[q & 1], static_cast<uint32_t>(q >> 1) & 1u, p.err, p.spin);
           __syncwarp();
           tc_fence_after();
           const uint32_t src = trow + (q & 1) * kWideAcc;
@@ -483,7 +483,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWideThreads<EPI>, 1
           if (lane == 0) mbar_arrive_cluster(acce_u32[q & 1]);
         }
       } else {
-        if (ok && !mbar_wait(&accf[q & 1], static_cast<uint32_t>(q >> 1) & 1u, p.err, p.spin)) ok = false;
+        if (ok) ok = warp_mbar_wait(&accf[q & 1], static_cast<uint32_t>(q >> 1) & 1u, p.err, p.spin);
         __syncwarp();
         tc_fence_after();
       }
