@@ -544,6 +544,13 @@ __global__ void __launch_bounds__(kThreadsA, 3) attention_kernel(const __grid_co
 // memory; the CTA that walks all blocks of a group combines them itself, a
 // group cut by the end of a share is combined by whichever CTA finishes last.
 //
+// A bounded wait that runs out: the compute warps go through the same units and
+// barriers, read at a unit's first barrier whether one of them gave up, and
+// leave together; they count the blocks that they owe to groups shared with
+// other CTAs, so that the counters return to zero.  The copying warp leaves
+// last, after its copies in flight have landed.  What the CTA had not finished
+// stays unwritten.
+//
 // Bound by HBM for many sequences.  Captured calls over 1500 frames, 20 heads,
 // nine rows, keys and values from HBM, against one CTA per group: 32 sequences
 // 55 -> 53 us, 96 sequences 137 -> 129 (5.9 TB/s), 16 sequences 31.3 -> 32.8
@@ -557,19 +564,15 @@ constexpr int kWkTiles = 3;
 struct WalkUnit {
   int row0, h, nq, blk;  // first query row, head, queries, key block
   int group, mine, qbuf, end;  // mine: blocks of the group this CTA walked when this is its last one (else 0)
+                               // end: the share's last unit
 };
 constexpr int kSmemWalk = 1024 + kWkTiles * kSmemK + 2 * kSmemQ + kWarps * kQG * 2 * 4 +
                           kWkTiles * static_cast<int>(sizeof(WalkUnit)) + (2 * kWkTiles + 4) * 8 + 16;
 
 __device__ __forceinline__ void compute_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-
-// A bounded wait; after a timeout the phase is still waited for (bounded), so
-// that no copy lands in a CTA that has exited.  False once even that ran out.
-__device__ __forceinline__ bool walk_wait(uint64_t *bar, uint32_t parity, uint32_t *err, long long limit) {
-  if (mbar_wait(bar, parity, err, limit)) return true;
-  mbar_drain(bar, parity);
-  return mbar_test(bar, parity) != 0;
-}
+// The CTA's end: the copying warp waits there for all others.
+__device__ __forceinline__ void walk_end_barrier() { asm volatile("bar.sync 2, 320;" ::: "memory"); }
+__device__ __forceinline__ void walk_end_arrive() { asm volatile("bar.arrive 2, 320;" ::: "memory"); }
 
 __global__ void __launch_bounds__(kWkThreads, 2)
     cross_walk_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -585,6 +588,9 @@ __global__ void __launch_bounds__(kWkThreads, 2)
   uint64_t *empty = full + kWkTiles;
   uint64_t *qfree = empty + kWkTiles;  // [2] every compute warp has read the queries
   int *s_last = reinterpret_cast<int *>(qfree + 2);
+  volatile int &s_gave_up = s_last[1];   // a compute warp's wait ran out
+  volatile int &s_counted = s_last[2];   // groups shared with other CTAs whose blocks here were counted
+  volatile int &s_arrivals = s_last[3];  // of the query warp on the tiles
 
   const int warp = warp_index(), lane = threadIdx.x & 31, tid = threadIdx.x;
   const int groups = p.n_seq * p.n_heads * p.qgroups;
@@ -601,6 +607,9 @@ __global__ void __launch_bounds__(kWkThreads, 2)
     }
     mbar_init(&qfree[0], kWarps);
     mbar_init(&qfree[1], kWarps);
+    s_gave_up = 0;
+    s_counted = 0;
+    for (int t = 0; t < kWkTiles; ++t) info[t] = WalkUnit{};
     fence_barrier_init();
     fence_proxy_async();
   }
@@ -629,12 +638,14 @@ __global__ void __launch_bounds__(kWkThreads, 2)
       // the acoustic memory is settled: nothing here waits for the previous kernel
       const uint32_t bytes = static_cast<uint32_t>(min(kKB, p.ctx)) * 128u;
       int slot_next = u < u_end ? __ldcg(p.seq_slot + g / p.qgroups / p.n_heads) : 0;  // read a group ahead
+      int n_copies = 0;
       for (; u < u_end && ok; ++g, blk = 0) {
         const int ih = g / p.qgroups, i = ih / p.n_heads, cache_row = slot_next * p.n_heads + ih - i * p.n_heads;
         bool ahead = false;
         for (; blk < p.n_chunks && u < u_end && ok; ++blk, ++u) {
           for (int kv = 0; kv < 2; ++kv) {
-            if (!(ok = walk_wait(&empty[tile], eph, p.err, spin))) break;
+            if (!(ok = warp_mbar_wait(&empty[tile], eph, p.err, spin))) break;
+            ++n_copies;
             if (elect_one()) {
               mbar_arrive_expect_tx(&full[tile], bytes);
               tma_load_3d(smem + tile * kSmemK, kv ? &tmV : &tmK, 0, blk * kKB, cache_row, &full[tile]);
@@ -647,8 +658,24 @@ __global__ void __launch_bounds__(kWkThreads, 2)
         }
       }
       pdl_wait();
-      if (ok) walk_wait(&empty[tile], eph, p.err, spin);
-      if (lane == 0) mbar_arrive_cta(&full[tile]);  // (the end, see below)
+      walk_end_barrier();
+      if (s_gave_up && lane == 0) {
+        // No copy lands in a CTA that has exited.  Nobody else looks at the
+        // tiles any more, so this warp makes up for arrivals of the query warp
+        // that did not come.
+        for (int c = max(0, n_copies - kWkTiles); c < n_copies; ++c) {
+          if (c >= s_arrivals) mbar_arrive_cta(&full[c % kWkTiles]);
+          mbar_drain(&full[c % kWkTiles], static_cast<uint32_t>(c / kWkTiles) & 1u);
+        }
+        // The blocks of shared groups (the first and the last of the share)
+        // that the compute warps did not come to count.
+        int counted = s_counted;
+        for (int q = u_begin / p.n_chunks; q * p.n_chunks < u_end; ++q) {
+          const int mine = min(u_end, (q + 1) * p.n_chunks) - max(u_begin, q * p.n_chunks);
+          if (mine == p.n_chunks || --counted >= 0) continue;
+          if (atomicAdd(&p.counters[q], mine) + mine == p.n_chunks) p.counters[q] = 0;
+        }
+      }
       return;
     }
     pdl_wait();  // the queries are the previous kernel's
@@ -667,7 +694,7 @@ __global__ void __launch_bounds__(kWkThreads, 2)
     };
     load_queries(g);
     WalkUnit w = {};
-    int n_groups = 0;
+    int n_groups = 0, n_arrivals = 0;
     for (; u < u_end && ok; ++g, blk = 0) {
       const int ih = g / p.qgroups, i = ih / p.n_heads, q0 = (g - ih * p.qgroups) * kQG;
       w.h = ih - i * p.n_heads;
@@ -675,11 +702,12 @@ __global__ void __launch_bounds__(kWkThreads, 2)
       w.row0 = i * p.rps + q0;
       w.group = g;
       for (int walked = 0; blk < p.n_chunks && u < u_end; ++blk, ++u) {
-        if (!(ok = walk_wait(&empty[tile], eph, p.err, spin))) break;
+        if (!(ok = warp_mbar_wait(&empty[tile], eph, p.err, spin))) break;
         if (walked++ == 0) {
           // ---- queries, pre-scaled by 1/8 = 1/sqrt(64) (exact in binary)
           w.qbuf = n_groups & 1;
-          if (!(ok = walk_wait(&qfree[w.qbuf], ((static_cast<uint32_t>(n_groups) >> 1) & 1u) ^ 1u, p.err, spin))) break;
+          if (!(ok = warp_mbar_wait(&qfree[w.qbuf], ((static_cast<uint32_t>(n_groups) >> 1) & 1u) ^ 1u, p.err, spin)))
+            break;
           ++n_groups;
           uint8_t *q = sQ + w.qbuf * kSmemQ;
 #pragma unroll
@@ -692,23 +720,24 @@ __global__ void __launch_bounds__(kWkThreads, 2)
           }
         }
         w.blk = blk;
+        w.end = u + 1 == u_end;
         w.mine = (blk == p.n_chunks - 1 || u + 1 == u_end) ? walked : 0;
         if (lane == 0) info[tile] = w;
         __syncwarp();
         if (lane == 0) mbar_arrive_cta(&full[tile]);  // unit and queries are in place
+        ++n_arrivals;
         next_tile();
         // the values' tile has nothing to add
-        if (!(ok = walk_wait(&empty[tile], eph, p.err, spin))) break;
+        if (!(ok = warp_mbar_wait(&empty[tile], eph, p.err, spin))) break;
         if (lane == 0) mbar_arrive_cta(&full[tile]);
+        ++n_arrivals;
         next_tile();
         if (walked == 1) load_queries(g + 1);
       }
     }
-    if (ok) walk_wait(&empty[tile], eph, p.err, spin);
-    if (lane == 0) {
-      info[tile].end = 1;
-      mbar_arrive_cta(&full[tile]);
-    }
+    if (lane == 0) s_arrivals = n_arrivals;
+    __syncwarp();
+    walk_end_arrive();
     return;
   }
 
@@ -724,13 +753,13 @@ __global__ void __launch_bounds__(kWkThreads, 2)
     }
   };
   pdl_wait();
-  while (true) {
-    if (!walk_wait(&full[tile], fph, p.err, spin)) break;
-    const WalkUnit w = info[tile];
-    if (w.end) break;
+  WalkUnit w;
+  do {
+    bool ok = warp_mbar_wait(&full[tile], fph, p.err, spin);  // (the same in all lanes)
+    w = info[tile];
     uint8_t *sK = smem + tile * kSmemK;
     const int key0 = w.blk * kKB;
-    const bool any = key0 + kw < p.ctx;  // this warp's slice has a visible key
+    const bool any = ok && key0 + kw < p.ctx;  // this warp's slice has a visible key
     float s[kNT][4];
     if (any) {
       const uint32_t q_u32 = smem_u32(sQ + w.qbuf * kSmemQ), k_u32 = smem_u32(sK);
@@ -750,7 +779,7 @@ __global__ void __launch_bounds__(kWkThreads, 2)
       }
     }
     __syncwarp();
-    if (lane == 0) {
+    if (ok && lane == 0) {
       mbar_arrive_cta(&empty[tile]);
       if (w.mine) mbar_arrive_cta(&qfree[w.qbuf]);
     }
@@ -797,8 +826,8 @@ __global__ void __launch_bounds__(kWkThreads, 2)
         lrow[r] += __shfl_xor_sync(0xffffffffu, lrow[r], 2);
       }
     }
-    if (!walk_wait(&full[tile], fph, p.err, spin)) break;
-    if (any) {
+    if (ok) ok = warp_mbar_wait(&full[tile], fph, p.err, spin);
+    if (any && ok) {
       // rows past the last frame become zeros, so P V adds exact zeros there
       const int z0 = p.ctx - key0 - kw;
       if (z0 < kKW) {
@@ -825,7 +854,10 @@ __global__ void __launch_bounds__(kWkThreads, 2)
         }
       }
     }
+    if (!ok) s_gave_up = 1;
     compute_barrier();  // every warp is done with the values, and with the last unit's sums
+    // (the same for all warps: none sets it for a later unit before the next barrier)
+    const int leave = s_gave_up;
     // stage this warp's (m, l, O) for the in-order combine: O over the values,
     // 8-float column groups XOR-swizzled by the row's low two bits
     float *so = reinterpret_cast<float *>(sV);
@@ -843,6 +875,7 @@ __global__ void __launch_bounds__(kWkThreads, 2)
         *reinterpret_cast<float2 *>(so + (warp * kQG + g + 8) * 64 + col) = make_float2(o[nd][2], o[nd][3]);
       }
     }
+    if (leave) break;
     compute_barrier();
 
     // ---- combine the warps in order (a warp without a visible key of the row
@@ -888,6 +921,7 @@ __global__ void __launch_bounds__(kWkThreads, 2)
       if (tid == 0) {
         __threadfence();
         const int last = atomicAdd(&p.counters[w.group], w.mine) + w.mine == p.n_chunks;
+        s_counted = s_counted + 1;
         if (last) {
           __threadfence();
           p.counters[w.group] = 0;
@@ -898,7 +932,8 @@ __global__ void __launch_bounds__(kWkThreads, 2)
       if (!*s_last) continue;
     }
     if (qi < w.nq) combine_blocks(pg + qi * kPartStride, p.n_chunks, d0, orow);
-  }
+  } while (!w.end);
+  walk_end_arrive();
 }
 
 // (cos, sin) of pos * base^(-2i/64) for every position below max_pos, or below

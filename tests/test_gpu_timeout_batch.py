@@ -1,7 +1,7 @@
 """Failure detection in the kernels that run several sequences (GPU): the
-bounded waits of the cluster split-K projections and of the pair kernel, split
-and unsplit (the output head), run out during one step, as in
-test_gpu_timeout.py, and the handle recovers.  Every copy and matrix
+bounded waits of the cluster split-K projections, of the pair kernel, split and
+unsplit (the output head), and of the walking cross-attention run out during
+one step, as in test_gpu_timeout.py, and the handle recovers.  Every copy and matrix
 instruction still completes; the waits only give up before it does, and the
 kernels then wait (bounded) for what they have in flight."""
 import numpy as np
@@ -63,3 +63,11 @@ def _timeout_and_recover(cfg, n, T, limits):
 @pytest.mark.parametrize("n,T", [(2, 0.0), (12, 0.0), (12, 0.8)])
 def test_projections_give_up_and_the_handle_recovers(n, T):
     _timeout_and_recover(syn.TINY, n, T, (32, 400))
+
+
+def test_the_walk_gives_up_and_its_counters_return_to_zero():
+    """52 sequences of 6 heads are two (sequence, head) groups per SM: walking
+    CTAs, most of whose shares cut a group that another CTA finishes.  A count
+    left behind by a CTA that gave up would merge that group too early, or
+    never, in the steps that follow."""
+    _timeout_and_recover(syn.TINY, 52, 0.0, (32, 400, 3000))
