@@ -539,6 +539,10 @@ __device__ __forceinline__ float key_value(uint32_t k) {
 // 2^-10 of the true one, so an id that scores best exactly is never more than
 // kRaceTol below the best estimate.
 constexpr float kRaceTol = 4e-3f;
+// That leaves 2e-3 for the rounding of two exact scores x - log(-log u), up to
+// two units in the last place of x: 1e-3 below 2^13.  A head's candidates lie
+// within 20 of its tile's maximum.
+constexpr float kRaceMaxX = 4096.f;
 constexpr float kLog2e = 1.4426950408889634f;
 __device__ __forceinline__ float neg_log2_estimate(float u) {
   const float t = 1.f - u;

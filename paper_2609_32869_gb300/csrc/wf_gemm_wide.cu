@@ -106,14 +106,17 @@ __device__ __forceinline__ void head_rows_greedy(const float4 (&z4)[R], uint32_t
 // exp(x) / -log(u), which needs three fast special functions per id; only ids
 // within kRaceTol of the warp's best are scored exactly (one lane, nearly
 // always), so the draw is that of the exact scores of every id.  (An id whose x is 20 below
-// the tile's maximum cannot win, as u lies in [2^-24, 1 - 2^-24], so the fast
-// exponential is good to 2^-20 wherever it matters.)
+// the tile's maximum cannot win, as u lies in [2^-24, 1 - 2^-24]; above that
+// the exponent's magnitude stays below 29 in base 2 and its four roundings make
+// the fast exponential good to 2^-17.)  The exact scores are rounded to fp32
+// themselves, two of them by up to two units in the last place of x together:
+// past |x| = kRaceMaxX every id is scored.
 // ss[k]: (slot and block row, step) of row k.
 template <int R>
 __device__ __forceinline__ void head_rows_sample(const GemmParams &p, const float4 (&z4)[R], uint32_t masked, int id0,
                                                  const int2 *ss, HeadRec (&r)[R]) {
   float z[R][4], u[R][4], e[R][4], w[R][4], zmax[R], sum[R];
-  const float c = __fdiv_rn(kLog2e, p.temperature);
+  const float c = fminf(__fdiv_rn(kLog2e, p.temperature), 3.402823466e38f);
 #pragma unroll
   for (int k = 0; k < R; ++k) {
     z[k][0] = masked & 1u ? -INFINITY : z4[k].x;
@@ -180,9 +183,9 @@ __device__ __forceinline__ void head_rows_sample(const GemmParams &p, const floa
   uint32_t more = 0;
 #pragma unroll
   for (int k = 0; k < R; ++k) {
-    // without a finite maximum every id is scored; a masked id scores -inf, so
-    // that a row without any other id has one
-    const bool all = !(fabsf(zmax[k]) <= 3.402823466e38f);
+    // without a maximum below kRaceMaxX every id is scored; a masked id scores
+    // -inf, so that a row without any other id has one
+    const bool all = !(fabsf(r[k].m) <= kRaceMaxX);
     const float floor = best[k] - best[k] * kRaceTol;
     cand[k] = masked;
     gid[k] = 0x7fffffff;
