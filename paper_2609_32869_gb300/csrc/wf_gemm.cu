@@ -16,7 +16,7 @@
 // a thread-block cluster; after the MMAs each pushes its fp32 partials over
 // distributed shared memory to the CTAs that finish the rows, which add them
 // in split order, so results are deterministic and independent of M, and no
-// partial ever travels through global memory.  Past kWideMinM rows the pushes
+// partial ever travels through global memory.  Past wide_min_rows() the pushes
 // (~16 bytes per cycle and SM) cost more than they save and pairs of SMs run
 // the projection instead (wf_gemm_wide.cu).
 //
@@ -47,16 +47,48 @@ constexpr int kMaxBT = 128;                // token rows per tile (MMA N)
 constexpr size_t kSmemPerSM = 228 * 1024;  // shared memory of one SM
 constexpr uint32_t kGroupBytes = 128 * 4 * 4;  // one split's partials of four token rows
 // Token rows above which pairs of SMs (wf_gemm_wide.cu) take a projection from
-// the cluster split-K.  Launches of a captured graph with weights from HBM, us
-// (cluster / pairs): 1280 x 1280 at 64, 96, 144 rows 6.3 / 7.8, 7.2 / 7.8,
-// 8.2 / 7.8; 1280 x 5120 9.8 / 13.9, 12.3 / 13.8, 15.6 / 13.9; 3840 x 1280 (30
-// weight tiles, so the pairs cover the GPU sooner) 7.7 / 7.5, 8.9 / 7.5,
-// 11.9 / 7.9; 5120 x 1280 8.2 / 7.7, 9.7 / 7.9, 12.9 / 8.4.  A step of 6
-// sequences (54 rows) takes 529 us with its wide projections on clusters, 514
-// on pairs.
+// the cluster split-K.  A pair goes through all of K for its tile, K / 64 steps
+// one after the other; a cluster shares K out and pays with pushes that grow
+// with the rows.  Many weight tiles let the pairs cover the GPU early.  A launch
+// of its own (no programmatic dependence) shows a pair's whole chain, so there
+// the line lies higher the longer K is and the fewer CTAs the clusters have in
+// all; behind a dependent launch the chain's weights are under way before the
+// previous kernel ends, and the line does not move.  Launches of a captured
+// graph, us (cluster / pairs), weights from HBM at the large widths, from L2 at
+// the tiny ones:
+//   3840 x 1280   45 rows  7.5 /  7.4   97 rows  9.7 /  7.6
+//   5120 x 1280   45 rows  8.0 /  7.7   97 rows 10.3 /  8.2
+//   2560 x 1280   72 rows  6.8 /  7.2   97 rows  7.8 /  7.3
+//   384 x 384     90 rows  5.3 /  5.4   97 rows  5.8 /  5.3  (1152, 1536 x 384 alike)
+//   1280 x 1280   97 rows  7.7 /  7.8  108 rows  7.7 /  7.8  126 rows  8.6 / 7.8
+//   1280 x 5120   97 rows 12.4 / 13.5  108 rows 13.2 / 13.5  126 rows 14.5 / 13.5
+//   1280 x 6400  108 rows 10.7 / 15.4  180 rows 12.7 / 15.4  252 rows 15.5 / 15.5
+//   384 x 1920    97 rows  7.3 /  9.1  180 rows  7.4 /  9.1  252 rows  8.6 / 9.1
+//   384 x 1536    97 rows  6.9 /  8.1  180 rows  6.5 /  8.2  252 rows  7.8 / 8.2
+//   768 x 3072   180 rows  9.2 / 10.4  216 rows 11.0 / 10.6  (clusters of 16)
+//   1024 x 4096   97 rows 11.3 / 11.9  126 rows 13.3 / 11.8  (128 CTAs)
+// A step of 12 sequences (108 rows, large widths, 4 layers) takes 656 us with a
+// lone launch's lines, 638 with 96; one of 20 (180 rows, tiny) 451 and 444.
 constexpr int kWideMinM = 96;
-constexpr int kWideMinMFewRows = 40;
+constexpr int kWideMinMFewRows = 40;  // many weight tiles
 constexpr int kWideFewRowsN = 3840;
+// lone launches: few weight tiles and a long K; a longer one whose clusters
+// leave SMs idle (two token tiles; clusters of 16 push most per row)
+constexpr int kWideMinMLongK = 112;
+constexpr int kWideLongKN = 1280;
+constexpr int kWideLongK = 1280;
+constexpr int kWideMinMRoom = 256;
+constexpr int kWideMinMRoom16 = 192;
+constexpr int kWideRoomK = 1536;
+constexpr int kWideRoomCtas = 104;
+
+static int wide_min_rows(int N, int K, int splits, bool pdl) {
+  if (N >= kWideFewRowsN) return kWideMinMFewRows;
+  if (pdl) return kWideMinM;
+  if (K >= kWideRoomK && (N + kBlockN - 1) / kBlockN * splits <= kWideRoomCtas)
+    return splits < 16 ? kWideMinMRoom : kWideMinMRoom16;
+  return N <= kWideLongKN && K >= kWideLongK ? kWideMinMLongK : kWideMinM;
+}
 
 // Epilogue of 16 consecutive token columns t0..t0+15 for output feature n.
 // acc[] holds the 16 accumulated values; every global load of the chunk (the
@@ -665,12 +697,12 @@ cudaError_t launch_gemm(const void *X, const void *W, GemmParams p, cudaStream_t
   if (quad && p.epi == EPI_KV && (p.N % 4 || p.q_cols % 4 || p.d_model % 4 || p.ld_out % 4))
     return cudaErrorInvalidValue;
   if (quad && p.epi == EPI_RESID && (p.tap0 || p.tap1) && p.ld_tap % 4) return cudaErrorInvalidValue;
-  // Past kWideMinM rows pairs of SMs on 256-row weight tiles (same bits).
+  // Past wide_min_rows() pairs of SMs on 256-row weight tiles (same bits).
   // They write four features at a time whatever the split, so a key/value
   // scatter with odd strides stays here.  They run the output head at any
   // number of rows.
   const bool quads = p.epi != EPI_KV || !(p.N % 4 || p.q_cols % 4 || p.d_model % 4 || p.ld_out % 4);
-  const int wide_m = p.N >= kWideFewRowsN ? kWideMinMFewRows : kWideMinM;
+  const int wide_m = wide_min_rows(p.N, p.K, std::max(1, p.splits), pdl);
   if (p.epi == EPI_HEAD || (p.M > wide_m && quads)) return launch_gemm_wide(X, W, p, s, pdl);
   size_t smem = 0;
   if (!plan_gemm(p, &smem)) return cudaErrorInvalidValue;
