@@ -1019,6 +1019,21 @@ cudaError_t attention_init() {
 // blocks, persistent CTAs walk even shares of all blocks (cross_walk_kernel,
 // with its measurements; it does not rotate, so a call with a RoPE table stays
 // with one CTA per group).  All do the same arithmetic in the same order.
+//
+// One CTA per group, three per SM, stays the better form over the acoustic
+// memory in two cases (us, one CTA per group / walking):
+//  - its only wave is nearly full (370-456 of 456 places): calls over 1500
+//    frames, 20 heads, 22 sequences of nine rows 34.6 / 41.1 (of 16, 70% full,
+//    29.5 / 32.5, 3 of them the clearing of counters that only a call pays for);
+//    a step, large widths, 4 layers: 22 sequences 708 / 722, 20 691 / 700, but 18
+//    679 / 675, 16 664 / 651 and, with a second wave begun, 24 794 / 751;
+//  - several query groups per head over keys and values that do not stay in L2:
+//    a walking CTA comes back to them for the next group when they are gone.
+//    Calls of 15 sequences of 33 rows 53.5 / 65.1, of 16 of 200 rows 228 / 270;
+//    prefill of 13 prompts of 33 tokens (100 MB of keys and values a layer) 1,150
+//    / 1,167; but calls of 10 of 33 rows (77 MB) 43.9 / 41.2.
+constexpr double kLoopWaveFill = 0.81;
+constexpr long long kWalkGroupsBytes = 88LL << 20;
 struct AttnForm {
   int n_sm, qgroups, n_chunks, cluster, loop, walk;
   bool counters() const { return n_chunks > 1 && !cluster && !loop; }  // the form counts finished blocks
@@ -1038,7 +1053,10 @@ static AttnForm attn_form(int n_seq, int rps, int n_heads, int ctx, int mode, bo
   const long long groups = static_cast<long long>(n_seq) * n_heads * f.qgroups;
   f.cluster = (f.n_chunks > 1 && f.n_chunks <= 8 && groups * f.n_chunks <= n_sm) ? 1 : 0;
   const bool many = !f.cluster && f.n_chunks > 1 && n_sm > 0 && groups >= 2LL * n_sm;
-  f.walk = (many && mode == 2 && !rope && groups * f.n_chunks <= 0x3fffffff) ? 1 : 0;
+  const long long places = 3LL * n_sm, kv_bytes = 256LL * n_seq * n_heads * ctx;
+  const bool full_wave = groups <= places && groups >= kLoopWaveFill * places;
+  const bool rereads = f.qgroups > 1 && kv_bytes > kWalkGroupsBytes;
+  f.walk = (many && mode == 2 && !rope && !full_wave && !rereads && groups * f.n_chunks <= 0x3fffffff) ? 1 : 0;
   f.loop = (many && !f.walk) ? 1 : 0;
   return f;
 }

@@ -81,3 +81,16 @@ def test_masked_frames_have_weight_zero(n_seq, rps, H, ctx, masked):
     assert torch.isfinite(big.float()).all()
     assert torch.equal(big, alone)
     np.testing.assert_allclose(ends, want, atol=2e-2, rtol=1e-2)
+
+
+# (sequences, rows, heads, frames): one CTA per group from 81% of a wave of
+# three CTAs on each of 152 SMs (370 of 456 groups) to a whole one, walking CTAs
+# on either side; two query groups over more and over less than 88 MiB of keys
+# and values
+@pytest.mark.parametrize("n_seq,rps,H,ctx", [(369, 3, 1, 300), (370, 3, 1, 300), (456, 3, 1, 300), (457, 3, 1, 300),
+                                             (13, 17, 20, 1500), (11, 17, 24, 1300), (16, 17, 15, 1500)])
+def test_forms_agree_where_they_change(n_seq, rps, H, ctx):
+    import torch
+    big, alone, ends, want = _calls(n_seq, rps, H, ctx, 0)
+    assert torch.equal(big, alone)
+    np.testing.assert_allclose(ends, want, atol=2e-2, rtol=1e-2)
