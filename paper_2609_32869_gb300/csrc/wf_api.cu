@@ -702,7 +702,6 @@ cudaError_t head(wf_handle *h, const float *x, const float2 *st, int stride, int
   GemmParams p = gemm_base(h, rows, h->V, h->d, EPI_HEAD);
   p.recs = recs;
   p.logits = (sampling || h->keep_logits) ? logits : nullptr;
-  p.keep_logits = h->keep_logits ? 1 : 0;
   p.temperature = sampling ? sp->temperature : 0.f;
   p.seed = sp ? sp->seed : 0;
   p.suppress = sp ? sp->d_suppress : nullptr;

@@ -511,14 +511,6 @@ __device__ __forceinline__ float word_to_uniform(uint32_t w) {
 __device__ __forceinline__ float word_to_open_uniform(uint32_t w) {
   return (static_cast<float>(w >> 9) + 0.5f) * (1.0f / 8388608.0f);
 }
-// Standard Gumbel noise for vocabulary id v of one (sequence, step, row, tag).
-__device__ __forceinline__ float gumbel(uint64_t seed, uint32_t seq, uint32_t step, uint32_t row,
-                                        uint32_t tag, uint32_t v) {
-  Philox4 o = philox4x32_10(v >> 2, row, step, (tag << 24) | (seq & 0xFFFFFFu),
-                            static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32));
-  const float u = word_to_open_uniform(o.x[v & 3]);
-  return -logf(-logf(u));
-}
 
 // Order-preserving key of a float; 0 (below every number) for NaN, and one
 // key for both zeros.

@@ -70,7 +70,6 @@ struct GemmParams {
   // EPI_HEAD
   HeadRec *recs;  // [M][n_tiles]
   float *logits;  // nullable [M][N] raw logits (sampling, or kept for inspection)
-  int keep_logits;
   float temperature;  // 0: greedy
   uint64_t seed;
   const uint8_t *suppress;
