@@ -1,7 +1,8 @@
 // Decode-time multi-head attention of a few query rows per sequence against a
 // per-sequence key/value cache laid out [slot][head][position][64] (bf16).
 //
-// One kernel serves the three attentions of the step:
+// attention_kernel serves the three attentions of the step (cross_walk_kernel,
+// below, the third one for many sequences):
 //  - mode 0, causal: the target's self-attention over its cache, query row j
 //    of a block starting at position L sees positions [0, L+j] (verify block,
 //    prompt, plain greedy step; Sec. 3.1 "one causal target pass");
@@ -11,7 +12,9 @@
 //  - mode 2, cross: all encoder frames (cross-attention, Sec. 3.2).
 //
 // A CTA takes one (sequence, head, group of <= 16 query rows, block of 256
-// keys).  Keys and values arrive as two TMA copies of 32 KB (the caches are
+// keys).  Keys and values arrive by TMA, a block of 32 KB at once from the
+// acoustic memory and 64 rows at a time, as many as hold a visible key, from a
+// text cache (the caches are
 // 3-D tensors (64, position, slot * heads), 128-byte swizzled in shared
 // memory; rows past the cache are zero-filled by the copy, value rows past
 // the visible keys are zeroed after it); each of the eight
@@ -42,7 +45,8 @@ constexpr int kKS = kKW / 16;         // 16-key steps per warp
 constexpr int kDPT = kQG * 64 / kThreadsA;  // output dims per thread in the combine
 constexpr int kPartStride = 2 + 64;   // m, l, o[64]
 // Scores are kept in base-2 units (times log2 e): every softmax weight, and
-// every weight of the merges of partial results, is one exp2.
+// every weight of the merges of partial results, is one exp2 (of the warps'
+// weights those below 2^-126 are taken as 0).
 constexpr int kSmemK = kKB * 128;     // bytes
 constexpr int kSmemQ = kQG * 128;
 // K, V, Q, then the warps' (m, l); the warps' O partials reuse the K tile.
@@ -1196,8 +1200,8 @@ extern "C" wf_status wf_attention(const void *d_q, const void *d_kc, const void 
 // library's module; make that first call before any stream capture.  All
 // calls share the array: calls that can overlap on the GPU (different
 // streams, or without ordering between them) race on it and must not be
-// issued.  The counters are cleared on every call; the partial sums need no
-// clearing.
+// issued.  The counters are cleared on every call of a form that counts
+// finished blocks; the partial sums need no clearing.
 namespace {
 constexpr size_t kNoAllocScratchBytes = size_t(8) << 20;  // 8 MiB
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];

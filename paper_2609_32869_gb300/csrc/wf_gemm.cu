@@ -8,8 +8,8 @@
 // <= 128) its N side.  Weight and token tiles stream into shared memory by
 // TMA (128-byte swizzle) through an mbarrier ring; one thread issues
 // tcgen05.mma into a TMEM accumulator; eight warps read it back with
-// tcgen05.ld for a fused epilogue (bias, GELU, residual add, taps, key/value
-// cache scatter, or the output-head reduction).
+// tcgen05.ld for a fused epilogue (bias, GELU, residual add, taps or key/value
+// cache scatter; the output head runs in wf_gemm_wide.cu).
 //
 // K is split into a fixed number of chunks per (N, K) shape so that ~150 CTAs
 // stream weights even for a single sequence.  The S split CTAs of a tile form
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kThreads) gemm_tc_kernel(const __grid_constant
   uint64_t *done = empty + stages;
   uint64_t *inbox_bar = done + 1;  // split-K: the partials of this CTA's token groups arrived
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 2);
-  // per-token (slot, position) for EPI_KV, (slot, step) for sampling heads
+  // per-token (slot, position) for EPI_KV
   int2 *tok = reinterpret_cast<int2 *>(smem + p.pipe_bytes + (2 * stages + 2) * 8 + 32);
   // split-K: where the partials of each group of four token rows go (the
   // cluster addresses of the slot and of its owner's inbox barrier)

@@ -2,8 +2,8 @@
 //
 // The skinny-M kernel of wf_gemm.cu gives every 128 x BT tile to one CTA; at
 // hundreds of rows each CTA then pulls its whole weight slab and token slab
-// through L2 for a small tile, and its split-K partials travel through tensor
-// memory.  Here two CTAs (one cluster) share a tile of 256 weight rows by BT
+// through L2 for a small tile, and the pushes of its split-K partials grow with
+// the rows.  Here two CTAs (one cluster) share a tile of 256 weight rows by BT
 // tokens: each holds its own 128 weight rows and half of the tokens in shared
 // memory, the even CTA issues one 256-row MMA for both, so a CTA fetches
 // 128 + BT/2 operand rows for 128 x BT outputs.  The grid is persistent (one
@@ -12,12 +12,23 @@
 // accumulators: eight epilogue warps work on one while the MMAs fill the
 // other.
 //
-// What bounds it: the copies' rate, ~85 bytes per cycle and SM (a 64-column
-// k-step of 128 weight rows and 16 token rows takes ~220 cycles whatever the
-// MMAs do; prefetching the weights into L2 first takes the same engine and
-// measured 5-15% slower).
-// Measured against wf_gemm.cu's folded split-K at 864 rows (one launch, cold):
-// out / cross out / fc2 36 -> 15 us on average, fc1 39 -> 23, QKV 37 -> 19,
+// What bounds it depends on the shape (clocks inside the kernel, cycles of 0.5
+// ns, means over the CTAs; 864 rows within a step of 96 sequences).  A launch
+// starts with ~2,700 to its first tile of operands and ends 4,000-5,000 after
+// its last MMA (TMEM reads, staging, stores); between them:
+//  - fc2, one tile of 80 k-steps: ~225 a step of 20 KB, the copies' rate of ~90
+//    bytes per cycle and SM; 16,000-18,000 of ~25,000 (prefetching the weights
+//    into L2 first takes the same engine and measured 5-15% slower);
+//  - out, cross out, cross query, 20 steps: ~6,500 of 14,000, so launch and
+//    epilogue weigh more than the copies;
+//  - fc1, two tiles a pair with GELU: 34,700, of them 11,300 in which the MMAs
+//    wait for the epilogue to free an accumulator, 4,400 for copies, and 12,000
+//    of epilogue after the last MMA;
+//  - acoustic K/V (24000 rows, 12 tiles a pair, 256 tokens): ~600 a step of 32 KB
+//    for 512 of MMAs; the MMAs wait for copies two thirds of the time, for the
+//    epilogue a tenth.
+// Measured against one CTA per tile that went through the chunks of its K in
+// turn, at 864 rows (one launch, cold): out / cross out / fc2 36 -> 15 us on average, fc1 39 -> 23, QKV 37 -> 19,
 // cross query 18 -> 11; acoustic K/V of 8 requests (12000 x 2560 x 1280)
 // 139 -> 75 us; 837 x 1280 x 5120 back to back 47 -> 18 us.  Stages of 128
 // columns instead of 64 (fewer barrier rounds, a shallower ring) measured 10%
@@ -671,9 +682,11 @@ static bool gemm_wide_plan(GemmParams &p, size_t *smem, int *pairs) {
   const bool direct = p.splits == 1 && (p.epi == EPI_KV || p.epi == EPI_F32 || p.epi == EPI_HEAD);
   const int max_bt = direct ? 256 : 128, n_nt = (p.N + 255) / 256, slots = n_sm / 2;
   // The token tile with the least estimated time: per tile the larger of its
-  // MMAs and its operand fetch (64 bytes per cycle and SM) over the k-steps
-  // plus an epilogue that grows with the tile, times the tiles of the busiest
-  // pair.
+  // MMAs and its operand fetch over the k-steps plus an epilogue that grows with
+  // the tile, times the tiles of the busiest pair.  The estimate only ranks the
+  // tiles of one shape (the choice is better than any single tile, see above): it
+  // leaves out what they share, takes 64 bytes per cycle and SM where an
+  // unhindered copy loop reaches ~90, and one epilogue for all kinds.
   long long best = 0;
   p.BT = 0;
   for (int bt = 32; bt <= max_bt; bt += 32) {
