@@ -326,13 +326,14 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_kernel(const __grid_cons
     if (C > 1) cluster_sync();  // every row has landed in every CTA
     else __syncthreads();
   } else {
-    op_ok = mbar_wait(&bar[1], 0, p.err, p.spin);
+    op_ok = warp_mbar_wait(&bar[1], 0, p.err, p.spin);
     if (!op_ok) *s_flag = 1;
   }
   // ---------------- MMAs: warp w takes the k-blocks [w kb / 8, (w + 1) kb / 8) of
   // every unit; within a k-block the k-steps alternate between two accumulators
   // (shorter dependency chains), added in a fixed order at the end
-  const bool landed = mbar_wait(&bar[0], 0, p.err, p.spin) && op_ok;
+  // (waits in front of MMAs have one answer per warp)
+  const bool landed = warp_mbar_wait(&bar[0], 0, p.err, p.spin) && op_ok;
   if (!landed) *s_flag = 1;
   float acc[U][2][4];
 #pragma unroll
@@ -647,8 +648,8 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_xattn_kernel(const __gri
       if (lane == 0 && t < M) sStat[t] = make_float2(mu, rsqrtf(var + p.ln_eps));
     }
   }
-  bool ok = mbar_wait(&bar[1], 0, p.err, spin);
-  ok = mbar_wait(&bar[0], 0, p.err, spin) && ok;
+  bool ok = warp_mbar_wait(&bar[1], 0, p.err, spin);
+  ok = warp_mbar_wait(&bar[0], 0, p.err, spin) && ok;
   if (!ok) *s_flag = 1;
 
   // ---------------- the 8 query columns: warp w over k-blocks [w kb / 8, (w + 1) kb / 8)
@@ -1030,8 +1031,8 @@ __global__ void __launch_bounds__(kSkThreads, 2) skinny_sattn_kernel(const __gri
       if (lane == 0 && t < M) sStat[t] = make_float2(mu, rsqrtf(var + p.ln_eps));
     }
   }
-  bool ok = mbar_wait(&bar[1], 0, p.err, spin);
-  ok = mbar_wait(&bar[0], 0, p.err, spin) && ok;
+  bool ok = warp_mbar_wait(&bar[1], 0, p.err, spin);
+  ok = warp_mbar_wait(&bar[0], 0, p.err, spin) && ok;
   if (!ok) *s_flag = 1;
 
   // ---------------- query, key and value columns: warp w over k-blocks [w kb / 8, (w + 1) kb / 8)

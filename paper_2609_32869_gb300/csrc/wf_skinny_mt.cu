@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kMtThreads, 2) skinny_mt_kernel(const __grid_c
       cp_async16(dst + 16u * i, p.resid + static_cast<size_t>(r_lo + r) * p.ld_resid + n_base + c);
     }
   }
-  bool ok = mbar_wait(wbar, 0, p.err, spin);
+  bool ok = warp_mbar_wait(wbar, 0, p.err, spin);  // (one answer per warp: MMAs hang on it)
   if (!ok) *s_flag = 1;
 
   // ---------------- MMAs: warp (wu, wt) owns the units of group wu and the
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kMtThreads, 2) skinny_mt_kernel(const __grid_c
                  z_addr = smem_u32(sZero);
   for (int q = 0; q < kb; ++q) {
     const int s = q % ns;
-    const bool landed = mbar_wait(&full[s], static_cast<uint32_t>(q / ns) & 1u, p.err, spin);
+    const bool landed = warp_mbar_wait(&full[s], static_cast<uint32_t>(q / ns) & 1u, p.err, spin);
     if (!landed) *s_flag = 1;
     if (ok && landed) {
       const uint32_t st = ring_base + s * L.stage_bytes;

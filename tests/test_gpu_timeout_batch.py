@@ -1,7 +1,8 @@
-"""Failure detection in the kernels that run several sequences (GPU): the
-bounded waits of the cluster split-K projections, of the pair kernel, split and
-unsplit (the output head), and of the walking cross-attention run out during
-one step, as in test_gpu_timeout.py, and the handle recovers.  Every copy and matrix
+"""Failure detection in the kernels of a step (GPU): the bounded waits of the
+warp-level projections (one sequence, or several by option), of the cluster
+split-K projections, of the pair kernel, split and unsplit (the output head),
+and of the walking cross-attention run out during one step, as in
+test_gpu_timeout.py, and the handle recovers.  Every copy and matrix
 instruction still completes; the waits only give up before it does, and the
 kernels then wait (bounded) for what they have in flight."""
 import numpy as np
@@ -21,7 +22,7 @@ def _steps(s, forced, sp):
     return out
 
 
-def _timeout_and_recover(cfg, n, T, limits):
+def _timeout_and_recover(cfg, n, T, limits, skinny=False):
     import torch
     from paper_2609_32869_gb300 import binding as B
     from paper_2609_32869_gb300.session import Session, upload_weights
@@ -34,6 +35,8 @@ def _timeout_and_recover(cfg, n, T, limits):
 
     def session():
         s = Session(cfg, dev, max_batch=n)
+        if skinny:
+            B.wf_set_option(s.h, B.WF_OPT_SKINNY, 1)
         s.prefill(slots, enc, prompt, np.full(n, 60, np.int32), sp=sp)
         return s
 
@@ -56,6 +59,11 @@ def _timeout_and_recover(cfg, n, T, limits):
         s.reset_slots(slots)
         assert s.compact() == n
     s.close()
+
+
+@pytest.mark.parametrize("n", [1, 5])
+def test_warp_level_projections_give_up_and_the_handle_recovers(n):
+    _timeout_and_recover(syn.TINY, n, 0.0, (32,), skinny=True)
 
 
 # 18 rows: cluster split-K; 108 rows: pairs of SMs (tiny widths, one chunk of
