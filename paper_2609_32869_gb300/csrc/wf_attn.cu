@@ -1120,6 +1120,15 @@ cudaError_t launch_rope_table(float2 *tab, int max_pos, float base, cudaStream_t
   return cudaGetLastError();
 }
 
+// Positions of a call's RoPE table: those of its cache, and over all frames
+// (mode 2, queries at positions 0..RPS-1) its queries' too.
+static int rope_rows(int mode, int rope, int RPS, int ctx) { return rope && mode == 2 && RPS > ctx ? RPS : ctx; }
+static size_t attn_scratch_bytes(int n_seq, int RPS, int n_heads, int ctx, int rope_rows) {
+  const size_t counters = static_cast<size_t>(attn_counter_slots(n_seq, RPS, n_heads)) * 4;
+  return attn_partial_floats(n_seq, RPS, n_heads, ctx) * sizeof(float) + ((counters + 255) / 256) * 256 +
+         static_cast<size_t>(rope_rows) * 32 * sizeof(float2) + 256;
+}
+
 // The kernel-level entry points: scratch holds the partials, the counters of
 // finished blocks and the RoPE table of the call's positions.  Counters are
 // cleared only for the form that counts; behind a table the attention is a
@@ -1151,8 +1160,9 @@ static wf_status attention_call(const void *d_q, const void *d_kc, const void *d
   if (rope) {
     float2 *tab = reinterpret_cast<float2 *>(static_cast<char *>(scratch) + pf * sizeof(float) +
                                              ((counters + 255) / 256) * 256);
-    rope_table_kernel<<<(ctx + kRopeRows - 1) / kRopeRows, 32 * kRopeRows, 0, s>>>(tab, ctx, rope_freq(rope_base), d_slot,
-                                                                                      d_base, mode == 2 ? 0 : n_seq, RPS);
+    const int rows = rope_rows(mode, rope, RPS, ctx);
+    rope_table_kernel<<<(rows + kRopeRows - 1) / kRopeRows, 32 * kRopeRows, 0, s>>>(
+        tab, rows, rope_freq(rope_base), d_slot, d_base, mode == 2 ? 0 : n_seq, RPS);
     if (cudaGetLastError() != cudaSuccess) return WF_ERR_CUDA;
     p.rope_tab = tab;
   }
@@ -1164,9 +1174,7 @@ static wf_status attention_call(const void *d_q, const void *d_kc, const void *d
 extern "C" size_t wf_attention_scratch_bytes(int32_t n_seq, int32_t RPS, int32_t n_heads,
                                              int32_t ctx) {
   if (n_seq <= 0 || RPS <= 0 || n_heads <= 0 || ctx <= 0) return 0;
-  const size_t counters = static_cast<size_t>(wf::attn_counter_slots(n_seq, RPS, n_heads)) * 4;
-  return wf::attn_partial_floats(n_seq, RPS, n_heads, ctx) * sizeof(float) +
-         ((counters + 255) / 256) * 256 + static_cast<size_t>(ctx) * 32 * sizeof(float2) + 256;
+  return wf::attn_scratch_bytes(n_seq, RPS, n_heads, ctx, wf::rope_rows(2, 1, RPS, ctx));
 }
 
 extern "C" wf_status wf_attention(const void *d_q, const void *d_kc, const void *d_vc,
@@ -1178,7 +1186,7 @@ extern "C" wf_status wf_attention(const void *d_q, const void *d_kc, const void 
       ctx <= 0 || mode < 0 || mode > 2)
     return WF_ERR_INVALID;
   if (mode != 2 && !d_base) return WF_ERR_INVALID;
-  if (scratch_bytes < wf_attention_scratch_bytes(n_seq, RPS, n_heads, ctx) || !d_scratch)
+  if (scratch_bytes < wf::attn_scratch_bytes(n_seq, RPS, n_heads, ctx, wf::rope_rows(mode, rope, RPS, ctx)) || !d_scratch)
     return WF_ERR_CAPACITY;
   if (wf::attention_init() != cudaSuccess) return WF_ERR_CUDA;
   return wf::attention_call(d_q, d_kc, d_vc, d_slot, d_base, n_seq, RPS, n_heads, ctx, mode, rope, rope_base, d_out,
@@ -1219,7 +1227,7 @@ extern "C" wf_status wf_attention_noalloc(const void *d_q, const void *d_kc, con
       ctx <= 0 || mode < 0 || mode > 2)
     return WF_ERR_INVALID;
   if (mode != 2 && !d_base) return WF_ERR_INVALID;
-  const size_t need = wf_attention_scratch_bytes(n_seq, RPS, n_heads, ctx);
+  const size_t need = wf::attn_scratch_bytes(n_seq, RPS, n_heads, ctx, wf::rope_rows(mode, rope, RPS, ctx));
   if (need > kNoAllocScratchBytes) return WF_ERR_CAPACITY;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return WF_ERR_CUDA;

@@ -94,3 +94,12 @@ def test_forms_agree_where_they_change(n_seq, rps, H, ctx):
     big, alone, ends, want = _calls(n_seq, rps, H, ctx, 0)
     assert torch.equal(big, alone)
     np.testing.assert_allclose(ends, want, atol=2e-2, rtol=1e-2)
+
+
+# more queries than frames: their positions run past the frames'
+@pytest.mark.parametrize("n_seq,rps,H,ctx", [(3, 209, 12, 42), (2, 300, 4, 257), (1, 17, 1, 1), (40, 65, 6, 64)])
+def test_queries_past_the_frames_rotate_by_their_positions(n_seq, rps, H, ctx):
+    import torch
+    big, alone, ends, want = _calls(n_seq, rps, H, ctx, 1)
+    assert torch.equal(big, alone)
+    np.testing.assert_allclose(ends, want, atol=2e-2, rtol=1e-2)
